@@ -94,6 +94,25 @@ PartPrep prep_of(const zeta_ctx* c, const Layout& L) {
   return q;
 }
 
+// Scratch of an assignment: the accumulator in the fields region; the grouped records in the rest of it
+// and in the regions delta_hat and spectra before it, which hold nothing yet.
+AssignScratch assign_scratch(const zeta_ctx* c, const Layout& L) {
+  AssignScratch a;
+  const size_t acc = sizeof(unsigned long long) * static_cast<size_t>(c->ng);
+  a.acc = at<unsigned long long>(c, L.fields);
+  a.small = at<double>(c, L.small);
+  a.counts = at<int>(c, L.counts);
+  a.tile_start = at<int64_t>(c, L.tstart);
+  const size_t rest = L.partials - L.fields - acc, before = L.fields - L.dhat;
+  char* const r0 = at<char>(c, L.fields + acc);
+  char* const b0 = at<char>(c, L.dhat);
+  a.tq = reinterpret_cast<float4*>(rest >= before ? r0 : b0);
+  a.tq_bytes = rest >= before ? rest : before;
+  a.cell = reinterpret_cast<int*>(rest >= before ? b0 : r0);
+  a.cell_bytes = rest >= before ? before : rest;
+  return a;
+}
+
 void drop_batch_graph(zeta_ctx* c) {
   if (c->batch_exec) cudaGraphExecDestroy(c->batch_exec);
   c->batch_exec = nullptr;
@@ -288,10 +307,8 @@ int zeta_assign(zeta_ctx* c, const float* particles, int64_t np, float* delta, d
   if (!particles || np < 1 || np > 0x7fffffffLL || !delta) return ZETA_EINVAL;
   ZK_TRY(need_ws(c, 0));
   const Layout L = layout(c, 0);
-  double* small = at<double>(c, L.small);
-  double* w = wsum ? wsum : small + kAssignScratchDoubles + 4;
-  return launch_assign(c, reinterpret_cast<const float4*>(particles), np, delta, w,
-                       at<unsigned long long>(c, L.fields), small, stream);
+  double* w = wsum ? wsum : at<double>(c, L.small) + kAssignScratchDoubles + 4;
+  return launch_assign(c, reinterpret_cast<const float4*>(particles), np, delta, w, assign_scratch(c, L), stream);
 }
 
 int zeta_fft_r2c(zeta_ctx* c, const float* delta, float* delta_hat, zeta_stream stream) {
@@ -397,14 +414,15 @@ int measure(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
   int64_t* tstart = at<int64_t>(c, L.tstart);
 
   const PartPrep q = prep_of(c, L);
-  if (want_p) {  // sort (and prepare) first; then the assignment is computed tile by tile
+  if (want_p) {  // sort (and prepare) first; the assignment then reads the prepared records
     ZK_TRY(launch_sort(c, parts, np, sorted, tstart, at<int>(c, L.counts), at<int>(c, L.orig), stream, nullptr, &q));
     if (!delta)
-      ZK_TRY(launch_assign_tiles(c, parts, np, tstart, q.s_cell, q.s_tq, dl, wsum, small, stream));
+      ZK_TRY(launch_assign_sorted(c, parts, np, q.s_cell, q.s_tq, dl, wsum,
+                                  reinterpret_cast<unsigned long long*>(fields), small, stream));
     else
       ZK_TRY(launch_wsum(c, parts, np, wsum, small, stream));
   } else if (!delta) {
-    ZK_TRY(launch_assign(c, parts, np, dl, wsum, reinterpret_cast<unsigned long long*>(fields), small, stream));
+    ZK_TRY(launch_assign(c, parts, np, dl, wsum, assign_scratch(c, L), stream));
   }
   ZK_TRY(launch_r2c(c, dl, dhat, stream));
   unsigned long long* hist = at<unsigned long long>(c, L.mhist);
@@ -493,11 +511,12 @@ int zeta_xi(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
     ZK_TRY(launch_sort(c, parts, np, at<float4>(c, L.sorted), tstart, at<int>(c, L.counts), at<int>(c, L.orig),
                        stream, nullptr, &q));
     if (!delta)
-      ZK_TRY(launch_assign_tiles(c, parts, np, tstart, q.s_cell, q.s_tq, dl, wsum, small, stream));
+      ZK_TRY(launch_assign_sorted(c, parts, np, q.s_cell, q.s_tq, dl, wsum,
+                                  reinterpret_cast<unsigned long long*>(fields), small, stream));
     else
       ZK_TRY(launch_wsum(c, parts, np, wsum, small, stream));
   } else if (!delta) {
-    ZK_TRY(launch_assign(c, parts, np, dl, wsum, reinterpret_cast<unsigned long long*>(fields), small, stream));
+    ZK_TRY(launch_assign(c, parts, np, dl, wsum, assign_scratch(c, L), stream));
   }
   ZK_TRY(launch_r2c(c, dl, dhat, stream));
   int f = 0;
@@ -526,10 +545,10 @@ int zeta_zeta_ell_ss(zeta_ctx* c, const float* data, int64_t nd, const float* ra
   double* small = at<double>(c, L.small);
   float* dd = at<float>(c, L.delta);
   float* dr = at<float>(c, L.dss);
-  unsigned long long* acc = at<unsigned long long>(c, L.fields);
+  const AssignScratch sc = assign_scratch(c, L);
   double* w = small + kAssignScratchDoubles + 4;
-  ZK_TRY(launch_assign(c, reinterpret_cast<const float4*>(data), nd, dd, w, acc, small, stream));
-  ZK_TRY(launch_assign(c, reinterpret_cast<const float4*>(randoms), nr, dr, w, acc, small, stream));
+  ZK_TRY(launch_assign(c, reinterpret_cast<const float4*>(data), nd, dd, w, sc, stream));
+  ZK_TRY(launch_assign(c, reinterpret_cast<const float4*>(randoms), nr, dr, w, sc, stream));
   ZK_TRY(launch_ss_fields(c, dd, dr, stream));
   ZK_TRY(measure(c, nullptr, 0, dd, forms, 0, 1, false, num, stream));
   return measure(c, nullptr, 0, dr, forms, 0, 1, false, den, stream);
@@ -671,7 +690,7 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
   int64_t* tstart = at<int64_t>(c, L.tstart);
   // representative data: this catalogue's fields for one (l, m)
   const PartPrep q = prep_of(c, L);
-  ZK_TRY(launch_assign(c, parts, np, dl, wsum, reinterpret_cast<unsigned long long*>(fields), small, stream));
+  ZK_TRY(launch_assign(c, parts, np, dl, wsum, assign_scratch(c, L), stream));
   ZK_TRY(launch_r2c(c, dl, dhat, stream));
   unsigned long long* hist = at<unsigned long long>(c, L.mhist);
   if (want_p) {
@@ -911,7 +930,7 @@ int zeta_backward_particles(zeta_ctx* c, const float* particles, int64_t np, con
   float* hfield = at<float>(c, L.hfield);
   float* direct = at<float>(c, L.direct);
   const size_t hbytes = sizeof(float) * c->ng * 4 * ((nb + 3) / 4);
-  ZK_TRY(launch_assign(c, parts, np, dl, wsum, reinterpret_cast<unsigned long long*>(fields), small, stream));
+  ZK_TRY(launch_assign(c, parts, np, dl, wsum, assign_scratch(c, L), stream));
   ZK_TRY(launch_r2c(c, dl, dhat, stream));
   ZK_TRY(launch_sort(c, parts, np, sorted, tstart, at<int>(c, L.counts), at<int>(c, L.orig), stream, sidx));
   if (cudaMemsetAsync(gk, 0, sizeof(float) * c->ng, stream) != cudaSuccess ||

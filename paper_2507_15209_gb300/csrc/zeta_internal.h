@@ -190,10 +190,21 @@ int launch_c2r_inplace(const zeta_ctx* c, float2* data, int nf, cudaStream_t s);
 int launch_primary(const zeta_ctx* c, const float2* dhat, float* out, cudaStream_t s);
 
 // ---- launchers (assign.cu) ----
+// acc: n^3 64-bit words; small: kAssignScratchDoubles; counts, tile_start: the tiling's; tq, cell: room
+// for the records grouped by tile (16 and 4 bytes a particle; used when it is enough)
+struct AssignScratch {
+  unsigned long long* acc = nullptr;
+  double* small = nullptr;
+  int* counts = nullptr;
+  int64_t* tile_start = nullptr;
+  float4* tq = nullptr;
+  int* cell = nullptr;
+  size_t tq_bytes = 0, cell_bytes = 0;
+};
 int launch_assign(const zeta_ctx* c, const float4* parts, int64_t np, float* delta, double* wsum,
-                  unsigned long long* acc, double* scratch2, cudaStream_t s);
+                  const AssignScratch& a, cudaStream_t s);
 int launch_wsum(const zeta_ctx* c, const float4* parts, int64_t np, double* wsum, double* scratch, cudaStream_t s);
-constexpr int kAssignScratchDoubles = 2 * 1024 + 4;
+constexpr int kAssignScratchDoubles = 2 * 1024 + 6;
 // Per-particle data computed once per catalogue with the float64 cell arithmetic, so the kernels
 // that run per (l, m) need none: the cell (linear index z n^2 + y n + x) and (t_x, t_y, t_z, w),
 // the in-cell offsets and the weight (0 for a non-finite particle).  o_*: original order
@@ -213,10 +224,9 @@ int launch_sort(const zeta_ctx* c, const float4* parts, int64_t np, float4* sort
 int launch_ss_fields(const zeta_ctx* c, float* data_delta, float* rand_delta, cudaStream_t s);
 // prepared data of an already sorted catalogue
 int launch_prep_sorted(const zeta_ctx* c, const float4* sorted, int64_t np, int* s_cell, float4* s_tq, cudaStream_t s);
-// assignment from the sorted, prepared catalogue (weight sums, then one CTA per tile writes delta)
-int launch_assign_tiles(const zeta_ctx* c, const float4* parts, int64_t np, const int64_t* tile_start,
-                        const int* s_cell, const float4* s_tq, float* delta, double* wsum, double* scratch,
-                        cudaStream_t s);
+// assignment from the sorted, prepared catalogue (acc: n^3 64-bit words of scratch)
+int launch_assign_sorted(const zeta_ctx* c, const float4* parts, int64_t np, const int* s_cell, const float4* s_tq,
+                         float* delta, double* wsum, unsigned long long* acc, double* scratch, cudaStream_t s);
 
 // ---- adjoint (adjoint.cu) ----
 // S: symmetrised loss weights of one l, device float [nb][nb]
