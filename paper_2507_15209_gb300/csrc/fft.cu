@@ -13,8 +13,6 @@
 // Every pass moves a tile of T contiguous complex columns (or RB rows) between HBM and
 // shared memory with coalesced accesses and transforms it with the radix-8 shared-memory
 // FFT of fft.cuh.
-#include <cuda_bf16.h>
-
 #include "fft.cuh"
 #include "fftreg.cuh"
 #include "zeta_internal.h"
@@ -65,12 +63,6 @@ __device__ __forceinline__ float ylm_dev(int l, int m, float nx, float ny, float
 }
 
 __device__ __forceinline__ int signed_freq(int i, int n) { return i < n / 2 ? i : i - n; }
-
-// two floats as a pair of bfloat16 (round to nearest even), the first in the low half
-__device__ __forceinline__ uint32_t bf16x2(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
 
 // ---------------------------------------------------------------------------------------
 // Threads per CTA of a register-staged transform: eight points per thread, at most MAXT.
@@ -171,22 +163,6 @@ __global__ void __launch_bounds__(256) k_c2r_x(float2* __restrict__ data, long l
   }
 }
 
-// e^{i pi j / 16} (j mod 16), from cos(a pi / 16), a = 0..8, written out; with j a compile-time
-// constant the factors become instruction operands.
-__device__ __forceinline__ float2 root32(int j) {
-  constexpr float c[9] = {1.0f,
-                          0.980785280403230449f,
-                          0.923879532511286756f,
-                          0.831469612302545237f,
-                          0.707106781186547524f,
-                          0.555570233019602225f,
-                          0.382683432365089772f,
-                          0.195090322016128268f,
-                          0.0f};
-  const int a = j & 15;
-  return make_float2(a <= 8 ? c[a] : -c[16 - a], a <= 8 ? c[8 - a] : c[a - 8]);
-}
-
 // x-pass of the field reconstruction: C2R of the rows of four fields at once, written as
 // one bin-interleaved group [z][y][x][4] (lane j = field 4g + j; missing fields give 0).
 // The half-length complex transform takes Z[k] = (X[k] + conj X[NC-k]) + i e^{2 pi i k/N}
@@ -283,6 +259,148 @@ __global__ void __launch_bounds__(RegThreads<N / 2, 4 * RB, 256>::NT)
       o[1] = make_float4(z0.y, z1.y, z2.y, z3.y);
     }
   }
+}
+
+// x-pass of the field reconstruction for grids of 256^3 and more: the same transform and arithmetic as
+// k_c2r_x4, arranged so that a thread's last butterfly is that of one row in all four fields.  It then
+// holds the four bins of a point and writes them directly, 32 contiguous bytes for two points, where
+// k_c2r_x4 gathers its outputs in shared memory and reads them back as bin groups.  The stages are
+// loops over butterflies, in place in shared memory (stage 0 reads global memory), XT threads, RB rows
+// of four fields per CTA (128 threads; 256 with twice the rows take 3933 us below).
+// Bound: HBM.  512^3, 20 fields: 4299 -> 3685 us (0.87 of the copy bandwidth); 256^3, 16 fields: 404 -> 389.
+__device__ __forceinline__ void store32(float* p, const float (&v)[8]) {  // 32 contiguous bytes, 32-byte aligned
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+
+template <int N, int XT>
+struct X4v {
+  static constexpr int NC = N / 2;
+  static constexpr int RB = XT / (NC / 8);  // rows per CTA
+  static constexpr size_t SMEM = (4 * RB * NC + StageTw<NC>::SIZE + 64) * sizeof(float2);
+};
+
+// Shared-memory position of point pos of transform col: rows of NC elements, the low four bits of the
+// position mixed with the upper ones so that the lanes of the second stage (64 apart) and of the last
+// (eight apart) hit distinct banks.
+template <int NC>
+__device__ __forceinline__ int x_slot(int pos, int col) {
+  const int d = NC == 256 ? (pos >> 6) & 1 : (pos >> 6);        // low bit of the stage-0 digit
+  const int e = NC == 256 ? (pos >> 7) & 1 : (pos >> 5) & 1;
+  return col * NC + (pos ^ (((pos >> 4) & 1) | (e << 1) | (d * 12)));
+}
+
+template <int N, int XT>
+__device__ __forceinline__ void x_stage0(const float2* __restrict__ src, long long fstride, int nfg, float2* ex,
+                                         const float2* tw, const float2* tww) {
+  using Y = X4v<N, XT>;
+  constexpr int NC = Y::NC, R0 = NC / 64, NT = 32 * 4 * Y::RB / XT;
+  // z_k = (X_k + conj X_{NC-k}) + i w (X_k - conj X_{NC-k}), w = conj(W_N^k), X_NC = 0
+  auto packw = [](float2 w, float2 xk, float2 xp) {
+    return cadd(cadd(xk, cconj(xp)), mul_i(cmul(w, csub(xk, cconj(xp)))));
+  };
+  const int u = threadIdx.x & 31;  // butterflies k = u and 64 - u (u = 0: 0 and 32): mirror-paired points
+  const int k0 = u, k1 = u == 0 ? 32 : 64 - u;
+  const float2 w0 = cconj(tww[k0]), w1 = cconj(tww[k1]);
+#pragma unroll 2
+  for (int i = 0; i < NT; ++i) {
+    const int col = (threadIdx.x >> 5) + i * (XT / 32);  // field col / RB, row col % RB
+    float2 a[R0], b[R0];
+    const float2* row = src + (col / Y::RB) * fstride + (col % Y::RB) * NC;
+    const bool have = col / Y::RB < nfg;
+#pragma unroll
+    for (int q = 0; q < R0; ++q) {
+      a[q] = have ? __ldcs(row + k0 + 64 * q) : make_float2(0.f, 0.f);
+      b[q] = have ? __ldcs(row + k1 + 64 * q) : make_float2(0.f, 0.f);
+    }
+    float2 x[R0], y[R0];
+#pragma unroll
+    for (int q = 0; q < R0; ++q) {
+      const float2 wa = q == 0 ? w0 : cmul(w0, root32(q * (16 / R0)));
+      const float2 wb = q == 0 ? w1 : cmul(w1, root32(q * (16 / R0)));
+      const float2 sa = q == 0 ? make_float2(0.f, 0.f) : a[R0 - q];
+      x[q] = packw(wa, a[q], u == 0 ? sa : b[R0 - 1 - q]);
+      y[q] = packw(wb, b[q], u == 0 ? b[R0 - 1 - q] : a[R0 - 1 - q]);
+    }
+    dft_small<R0, true>(x);
+    twiddle<R0, NC, true>(x, k0, tw);
+    dft_small<R0, true>(y);
+    twiddle<R0, NC, true>(y, k1, tw);
+#pragma unroll
+    for (int p = 0; p < R0; ++p) {
+      ex[x_slot<NC>(k0 + 64 * p, col)] = x[p];
+      ex[x_slot<NC>(k1 + 64 * p, col)] = y[p];
+    }
+  }
+}
+template <int N, int XT>
+__device__ __forceinline__ void x_stage1(float2* ex, const float2* tw) {
+  using Y = X4v<N, XT>;
+  constexpr int NC = Y::NC, PER = NC / 8, NT = PER * 4 * Y::RB / XT;
+  const int k = threadIdx.x % PER, j = k & 7, b = (k >> 3) * 64 + j;
+#pragma unroll 2
+  for (int i = 0; i < NT; ++i) {
+    const int col = threadIdx.x / PER + i * (XT / PER);
+    float2 x[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) x[a] = ex[x_slot<NC>(b + 8 * a, col)];
+    dft_small<8, true>(x);
+    twiddle<8, 64, true>(x, j, tw + StageTw<NC>::off(1));
+#pragma unroll
+    for (int a = 0; a < 8; ++a) ex[x_slot<NC>(b + 8 * a, col)] = x[a];
+  }
+}
+template <int N, int XT, bool BF16>
+__device__ __forceinline__ void x_stage2(const float2* ex, float* __restrict__ out) {
+  using Y = X4v<N, XT>;
+  constexpr int NC = Y::NC, R0 = NC / 64, KAP = NC / 8;
+  static_assert(KAP * Y::RB == XT, "one butterfly of four fields per thread");
+  const int r = threadIdx.x / KAP, lam = threadIdx.x % KAP;  // lam: index of the first output, lanes along x
+  const int kap = (lam % R0) * 8 + lam / R0;
+  float2 x[4][8];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[f][q] = ex[x_slot<NC>(8 * kap + q, f * Y::RB + r)];
+    dft_small<8, true>(x[f]);
+  }
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int at = r * N + 2 * (lam + 8 * R0 * p);  // point within the task's rows
+    if constexpr (BF16) {  // four bins of a point as bfloat16 (8 bytes), rounded to nearest even
+      uint4 o;
+      o.x = bf16x2(x[0][p].x, x[1][p].x);
+      o.y = bf16x2(x[2][p].x, x[3][p].x);
+      o.z = bf16x2(x[0][p].y, x[1][p].y);
+      o.w = bf16x2(x[2][p].y, x[3][p].y);
+      *reinterpret_cast<uint4*>(reinterpret_cast<uint2*>(out) + at) = o;
+    } else {
+      const float o[8] = {x[0][p].x, x[1][p].x, x[2][p].x, x[3][p].x, x[0][p].y, x[1][p].y, x[2][p].y, x[3][p].y};
+      store32(out + 4 * static_cast<size_t>(at), o);
+    }
+  }
+}
+
+template <int N, int XT, bool BF16>
+__global__ void __launch_bounds__(XT, 768 / XT)
+    k_c2r_x4v(const float2* __restrict__ spec, long long fstride, int nf, float* __restrict__ out,
+              const float2* __restrict__ twg) {
+  using Y = X4v<N, XT>;
+  constexpr int NC = Y::NC;
+  extern __shared__ float2 sm[];
+  float2* tw = sm + 4 * Y::RB * NC;            // per-stage twiddles
+  float2* tww = tw + StageTw<NC>::SIZE;  // W_N^k, k < 64
+  stage_tw_fill<NC>(tw, twg, 2);
+  for (int i = threadIdx.x; i < 64; i += XT) tww[i] = twg[i];
+  __syncthreads();
+  const int g = blockIdx.y;
+  const long long r0 = static_cast<long long>(blockIdx.x) * Y::RB;
+  x_stage0<N, XT>(spec + 4 * g * fstride + r0 * NC, fstride, nf - 4 * g < 4 ? nf - 4 * g : 4, sm, tw, tww);
+  __syncthreads();
+  x_stage1<N, XT>(sm, tw);
+  __syncthreads();
+  x_stage2<N, XT, BF16>(sm, out + (static_cast<long long>(g) * N * N + r0) * N * (BF16 ? 2 : 4));
 }
 
 // z-pass of the field reconstruction with the multipole window fused in.
@@ -500,6 +618,7 @@ constexpr int kTz = 8;   // columns per z-pass (window) tile
 constexpr int kTy = 16;  // columns per plain pencil tile
 constexpr int kRB = 8;   // rows per x-pass tile
 constexpr int kRB4 = 4;  // rows per four-field x-pass tile
+constexpr int kX4Threads = 128;  // threads of the direct-store x-pass
 
 template <typename K>
 int set_smem(K kernel, size_t bytes) {
@@ -587,6 +706,22 @@ int alm_x_pass(const zeta_ctx* c, int nf, const float2* spec, float* out, cudaSt
   StageScope prof(c, ST_ALM_X, 1, s);
   const size_t smx = x4_smem<N, RB>();
   const int ng4 = (nf + 3) / 4;
+  // k_c2r_x4 remains for its narrow shape, for smaller grids and for fields on 16-byte boundaries only
+  if constexpr (N >= 256 && RB == kRB4) {
+    if (bf16 || (reinterpret_cast<uintptr_t>(out) & 31) == 0) {  // its stores are 32 bytes wide
+      constexpr int XT = kX4Threads;
+      using Y = X4v<N, XT>;
+      const dim3 grid(N * N / Y::RB, ng4);
+      if (bf16) {
+        if (set_smem(k_c2r_x4v<N, XT, true>, Y::SMEM)) return ZETA_ECUDA;
+        k_c2r_x4v<N, XT, true><<<grid, XT, Y::SMEM, s>>>(spec, fstride, nf, out, c->d_tw);
+      } else {
+        if (set_smem(k_c2r_x4v<N, XT, false>, Y::SMEM)) return ZETA_ECUDA;
+        k_c2r_x4v<N, XT, false><<<grid, XT, Y::SMEM, s>>>(spec, fstride, nf, out, c->d_tw);
+      }
+      return check_launch();
+    }
+  }
   if (bf16) {
     if (set_smem(k_c2r_x4<N, RB, true>, smx)) return ZETA_ECUDA;
     k_c2r_x4<N, RB, true><<<dim3(N * N / RB, ng4), RegThreads<N / 2, 4 * RB, 256>::NT, smx, s>>>(

@@ -19,9 +19,35 @@
 // The exchange buffer may be padded by PADR elements every PADR points (PADR = 0: none),
 // which keeps the last stage of narrow (T = 8) pencils free of bank conflicts.
 #pragma once
+#include <cuda_bf16.h>
+
+#include <cstdint>
+
 #include "fft.cuh"
 
 namespace zk {
+
+// two floats as a pair of bfloat16 (round to nearest even), the first in the low half
+__device__ __forceinline__ uint32_t bf16x2(float a, float b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// e^{i pi j / 16} (j mod 16), from cos(a pi / 16), a = 0..8, written out; with j a compile-time
+// constant the factors become instruction operands.
+__device__ __forceinline__ float2 root32(int j) {
+  constexpr float c[9] = {1.0f,
+                          0.980785280403230449f,
+                          0.923879532511286756f,
+                          0.831469612302545237f,
+                          0.707106781186547524f,
+                          0.555570233019602225f,
+                          0.382683432365089772f,
+                          0.195090322016128268f,
+                          0.0f};
+  const int a = j & 15;
+  return make_float2(a <= 8 ? c[a] : -c[16 - a], a <= 8 ? c[8 - a] : c[a - 8]);
+}
 
 template <int L>
 __host__ __device__ constexpr int plan_radix(int s) {
