@@ -9,6 +9,7 @@
 //                   k-space; dL/dx_p = direct + (N_g w_p / W) grad(interpolated dL/d delta).
 // The particle scatter uses float atomics, so those gradients are reproducible only to float32
 // rounding; everything else is order-fixed.
+#include "cell.cuh"
 #include "zeta_internal.h"
 
 namespace zk {
@@ -36,7 +37,8 @@ __device__ __forceinline__ void bs_w(float t, float* w, float* dw) {
   }
 }
 
-__device__ __forceinline__ int cell_t(float x, double inv_h, int n, float& t) {
+// The float64 formula of a coordinate's cell and offset, for what the integer form does not take (cell.cuh).
+__device__ __noinline__ int cell_f64(float x, double inv_h, int n, float& t) {
   const double u = static_cast<double>(x) * inv_h;
   const double v = u - floor(u / n) * n;
   int c = static_cast<int>(floor(v));
@@ -46,54 +48,106 @@ __device__ __forceinline__ int cell_t(float x, double inv_h, int n, float& t) {
   if (t >= 1.f) t = 0.99999994f;
   return c;
 }
+__device__ __forceinline__ int cell_t(float x, const CellScale& cs, int n, float& t) {
+  int c;
+  return cell_int(x, cs, n, c, t) ? c : cell_f64(x, cs.inv_h, n, t);
+}
 
+// q += sum S a a and the fields replaced by h = 2 delta S a, two points per thread so that each float4 of S
+// read from shared memory serves eight multiply-adds.  Bound: HBM (fields read and
+// written) and shared-memory reads.  256^3, 10 bins: 550 us, 3.3 TB/s.
 template <int NBP>
 __global__ void __launch_bounds__(kAT) k_adj_node(const float* __restrict__ delta, float4* __restrict__ f4, long long ng,
                                                   int nb, const float* __restrict__ S, float* __restrict__ q) {
-  constexpr int G = NBP / 4;
-  __shared__ float s_s[NBP * NBP];
+  constexpr int G = NBP / 4, P = 2;
+  __shared__ __align__(16) float s_s[NBP * NBP];
   for (int i = threadIdx.x; i < NBP * NBP; i += blockDim.x) {
     const int r = i / NBP, c = i % NBP;
     s_s[i] = (r < nb && c < nb) ? S[r * nb + c] : 0.f;
   }
   __syncthreads();
-  const int ngrp = (nb + 3) / 4;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < ng;
-       i += static_cast<long long>(blockDim.x) * gridDim.x) {
-    float a[NBP];
+  // ng is a multiple of P kAT (n >= 16)
+  for (long long i0 = blockIdx.x * static_cast<long long>(P * kAT) + threadIdx.x; i0 < ng;
+       i0 += static_cast<long long>(P * kAT) * gridDim.x) {
+    float a[P][NBP], d[P], qs[P];
 #pragma unroll
+    for (int u = 0; u < P; ++u) {
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const float4 v = f4[g * ng + i0 + u * kAT];
+        a[u][4 * g] = v.x;
+        a[u][4 * g + 1] = v.y;
+        a[u][4 * g + 2] = v.z;
+        a[u][4 * g + 3] = v.w;
+      }
+      d[u] = 2.f * delta[i0 + u * kAT];
+      qs[u] = 0.f;
+    }
+#pragma unroll 1
     for (int g = 0; g < G; ++g) {
-      const float4 v = (g < ngrp) ? f4[g * ng + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-      a[4 * g] = v.x;
-      a[4 * g + 1] = v.y;
-      a[4 * g + 2] = v.z;
-      a[4 * g + 3] = v.w;
+      float h[P][4];
+      float4 own[P];  // this group's values once more (a itself is indexed by constants only)
+#pragma unroll
+      for (int u = 0; u < P; ++u) own[u] = f4[g * ng + i0 + u * kAT];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int b = 4 * g + j;
+        float t[P];
+#pragma unroll
+        for (int u = 0; u < P; ++u) t[u] = 0.f;
+#pragma unroll
+        for (int g2 = 0; g2 < G; ++g2) {
+          const float4 sv = *reinterpret_cast<const float4*>(s_s + b * NBP + 4 * g2);
+#pragma unroll
+          for (int u = 0; u < P; ++u) {
+            t[u] = fmaf(sv.x, a[u][4 * g2], t[u]);
+            t[u] = fmaf(sv.y, a[u][4 * g2 + 1], t[u]);
+            t[u] = fmaf(sv.z, a[u][4 * g2 + 2], t[u]);
+            t[u] = fmaf(sv.w, a[u][4 * g2 + 3], t[u]);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < P; ++u) {
+          qs[u] = fmaf(j == 0 ? own[u].x : j == 1 ? own[u].y : j == 2 ? own[u].z : own[u].w, t[u], qs[u]);
+          h[u][j] = d[u] * t[u];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < P; ++u) f4[g * ng + i0 + u * kAT] = make_float4(h[u][0], h[u][1], h[u][2], h[u][3]);
     }
-    const float d = delta[i];
-    float qs = 0.f;
-    float h[NBP];
 #pragma unroll
-    for (int b = 0; b < NBP; ++b) {
-      float t = 0.f;
-#pragma unroll
-      for (int b2 = 0; b2 < NBP; ++b2) t = fmaf(s_s[b * NBP + b2], a[b2], t);
-      qs = fmaf(a[b], t, qs);
-      h[b] = 2.f * d * t;
-    }
-    q[i] += qs;
-#pragma unroll
-    for (int g = 0; g < G; ++g)
-      if (g < ngrp) f4[g * ng + i] = make_float4(h[4 * g], h[4 * g + 1], h[4 * g + 2], h[4 * g + 3]);
+    for (int u = 0; u < P; ++u) q[i0 + u * kAT] += qs[u];
   }
 }
 
-// gk(n) -= 2 Mhat(n) delta_hat(n) (2l+1)/(4 pi) sum_bb' S[b,b'] T_b(n) T_b'(n), non-Nyquist modes
-__global__ void __launch_bounds__(kAT) k_adj_mass(const float2* __restrict__ dhat, const float* __restrict__ jt, int nbp,
-                                                  const float* __restrict__ mhat, int n, int nb, const float* __restrict__ S,
-                                                  float coef, float2* __restrict__ gk) {
-  __shared__ float s_s[kMaxBins * kMaxBins];
-  for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) s_s[i] = S[i];
+// The uniform term's share of gk: gk(n) -= 2 Mhat(n) delta_hat(n) sum_l (2l+1)/(4 pi) sum_bb' S_l[b,b'] T_lb(n)
+// T_lb'(n) over the non-Nyquist modes.  The sum over l and bins depends on the mode only through |n|^2, so it
+// is formed once per value of |n|^2 and the modes are visited once (256^3, 7 multipoles, 10 bins:
+// 7 x 2179 us with the sums per mode and multipole, 56 us in all now).
+__global__ void __launch_bounds__(kAT) k_adj_mass_table(const float* __restrict__ jt, long long nn2, int nbp, int nb,
+                                                        int lmax, const float* __restrict__ S, float* __restrict__ tab) {
+  extern __shared__ float s_s[];  // [lmax + 1][nb][nb]
+  for (int i = threadIdx.x; i < (lmax + 1) * nb * nb; i += blockDim.x) s_s[i] = S[i];
   __syncthreads();
+  const long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
+  if (i >= nn2) return;
+  float sum = 0.f;
+  for (int l = 0; l <= lmax; ++l) {
+    const float* t = jt + (l * nn2 + i) * nbp;
+    const float* sl = s_s + l * nb * nb;
+    float c = 0.f;
+    for (int b = 0; b < nb; ++b) {
+      float r = 0.f;
+      for (int b2 = 0; b2 < nb; ++b2) r = fmaf(sl[b * nb + b2], __ldg(t + b2), r);
+      c = fmaf(__ldg(t + b), r, c);
+    }
+    sum = fmaf(2.f * (2.f * l + 1.f) / 12.566370614359172f, c, sum);
+  }
+  tab[i] = sum;
+}
+
+__global__ void __launch_bounds__(kAT) k_adj_mass(const float2* __restrict__ dhat, const float* __restrict__ tab,
+                                                  const float* __restrict__ mhat, int n, float2* __restrict__ gk) {
   const int nc = n / 2;
   const long long total = static_cast<long long>(n) * n * nc;
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
@@ -102,159 +156,161 @@ __global__ void __launch_bounds__(kAT) k_adj_mass(const float2* __restrict__ dha
               iz = static_cast<int>(i / (static_cast<long long>(nc) * n));
     if (iy == n / 2 || iz == n / 2) continue;
     const int fy = iy < n / 2 ? iy : iy - n, fz = iz < n / 2 ? iz : iz - n;
-    const long long n2 = static_cast<long long>(ix) * ix + fy * fy + fz * fz;
-    const float* tb = jt + n2 * nbp;
-    float c = 0.f;
-    for (int b = 0; b < nb; ++b) {
-      float t = 0.f;
-      for (int b2 = 0; b2 < nb; ++b2) t = fmaf(s_s[b * nb + b2], __ldg(tb + b2), t);
-      c = fmaf(__ldg(tb + b), t, c);
-    }
-    const float f = 2.f * coef * c * mhat[ix] * mhat[iy] * mhat[iz];
-    const float2 d = dhat[i];
-    gk[i] = make_float2(gk[i].x - f * d.x, gk[i].y - f * d.y);
+    const float f = __ldg(tab + (ix * ix + fy * fy + fz * fz)) * (mhat[ix] * mhat[iy] * mhat[iz]);
+    const float2 d = dhat[i], g = gk[i];
+    gk[i] = make_float2(g.x - f * d.x, g.y - f * d.y);
   }
 }
 
-// Particle adjoint: persistent CTAs over tiles, batches of kAPB particles.
-// particles per batch: keeps the static shared memory of a CTA under 48 KB
-template <int NBP>
-struct AdjBatch {
-  static constexpr int APB = NBP >= 24 ? 64 : 128;
-};
-
+// Particle adjoint.  A warp takes eight particles of the tile-sorted catalogue, four lanes each, and keeps
+// everything in registers, without a barrier: the lanes of a particle hold the four nodes along x of every
+// stencil row (D = 4; for D = 2 the four nodes of a z-layer), so a gather and an atomic of a row each cover
+// 64 contiguous bytes.  Per bin group the lanes sum w v and the parts of its gradient over their nodes, then
+// reduce-scatter: lane i holds f and grad f of bin 4 g + i.  c = (2 w_p / W) S f takes f from the other
+// lanes by shuffles; the direct term sum_b c_b grad f_b is added to the particle's slot; and c is
+// scattered with the assignment stencil by float4 atomics.  Bound: L2 atomics and gathers.  256^3, 1M
+// particles, 10 bins, D = 4: 2167 us with one thread per particle and bin group (values and gradients
+// through shared memory), 974 us now.
 template <int NBP, int D>
-__global__ void __launch_bounds__(kAT)
-    k_adj_points(const float4* __restrict__ sorted, const long long* __restrict__ tile_start,
-                 const int* __restrict__ sidx, const float4* __restrict__ f4, long long ng, int n, int nb, double inv_h,
+__global__ void __launch_bounds__(kAT, 2)
+    k_adj_points(const int* __restrict__ s_cell, const float4* __restrict__ s_tq, const int* __restrict__ sidx,
+                 long long np, const float4* __restrict__ f4, long long ng, int n, int nb, float hinv,
                  const float* __restrict__ S, const double* __restrict__ wsum, float4* __restrict__ h4,
                  float* __restrict__ direct) {
-  constexpr int OFF = D / 2 - 1;
-  constexpr int kAPB = AdjBatch<NBP>::APB;
-  __shared__ float s_s[NBP * NBP];
-  __shared__ int4 org[kAPB];
-  __shared__ float bw[kAPB][6 * D];    // wx, wy, wz, dwx, dwy, dwz (derivatives already / H)
-  __shared__ float fv[kAPB][NBP];      // f_b, then c_b
-  __shared__ float gv[kAPB][NBP][3];   // grad f_b
-  __shared__ float pw[kAPB];
+  constexpr int OFF = D / 2 - 1, G = NBP / 4;
+  __shared__ __align__(16) float s_s[NBP * NBP];
   for (int i = threadIdx.x; i < NBP * NBP; i += blockDim.x) {
     const int r = i / NBP, c = i % NBP;
     s_s[i] = (r < nb && c < nb) ? S[r * nb + c] : 0.f;
   }
+  __syncthreads();
   const float wscale = static_cast<float>(2.0 / wsum[0]);
-  const float hinv = static_cast<float>(inv_h);
-  const int ngrp = (nb + 3) / 4;
-  const int nt = n / kTile;
-  const long long ntiles = static_cast<long long>(nt) * nt * nt;
-  const int mask = n - 1;
-  // full batches of kAPB consecutive particles of the tile-sorted catalogue (a tile holds few
-  // particles at galaxy-catalogue densities; consecutive tiles keep the batch's stencils close together)
-  const long long ptot = tile_start[ntiles];
-  {
-    for (long long bs = static_cast<long long>(blockIdx.x) * kAPB; bs < ptot;
-         bs += static_cast<long long>(gridDim.x) * kAPB) {
-      const int cnt = static_cast<int>((ptot - bs) < kAPB ? (ptot - bs) : kAPB);
-      __syncthreads();
-      if (threadIdx.x < cnt) {
-        const int me = threadIdx.x;
-        const float4 pp = sorted[bs + me];
-        float tx, ty, tz;
-        const int cx = cell_t(pp.x, inv_h, n, tx), cy = cell_t(pp.y, inv_h, n, ty), cz = cell_t(pp.z, inv_h, n, tz);
-        float w[D], dw[D];
-        bs_w<D>(tx, w, dw);
-        for (int o = 0; o < D; ++o) {
-          bw[me][o] = w[o];
-          bw[me][3 * D + o] = dw[o] * hinv;
-        }
-        bs_w<D>(ty, w, dw);
-        for (int o = 0; o < D; ++o) {
-          bw[me][D + o] = w[o];
-          bw[me][4 * D + o] = dw[o] * hinv;
-        }
-        bs_w<D>(tz, w, dw);
-        for (int o = 0; o < D; ++o) {
-          bw[me][2 * D + o] = w[o];
-          bw[me][5 * D + o] = dw[o] * hinv;
-        }
-        org[me] = make_int4(cx - OFF, cy - OFF, cz - OFF, 0);
-        pw[me] = (isfinite(pp.w) && isfinite(pp.x) && isfinite(pp.y) && isfinite(pp.z)) ? pp.w : 0.f;
-      }
-      __syncthreads();
-      // values and gradients of every field group at every particle of the batch
-      for (int task = threadIdx.x; task < cnt * ngrp; task += blockDim.x) {
-        const int p = task % cnt, g = task / cnt;
-        const int4 o = org[p];
-        const float* w = bw[p];
-        const float4* base = f4 + g * ng;
-        float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), gx = v0, gy = v0, gz = v0;
-        for (int oz = 0; oz < D; ++oz) {
-          const long long zrow = static_cast<long long>((o.z + oz) & mask) * n;
-          for (int oy = 0; oy < D; ++oy) {
-            const float4* row = base + (zrow + ((o.y + oy) & mask)) * n;
-            const float wyz = w[2 * D + oz] * w[D + oy];
-            const float dy = w[2 * D + oz] * w[4 * D + oy];
-            const float dz = w[5 * D + oz] * w[D + oy];
-            for (int ox = 0; ox < D; ++ox) {
-              const float4 v = __ldg(row + ((o.x + ox) & mask));
-              const float a = wyz * w[ox], ax = wyz * w[3 * D + ox], ay = dy * w[ox], az = dz * w[ox];
-              v0.x = fmaf(a, v.x, v0.x); v0.y = fmaf(a, v.y, v0.y); v0.z = fmaf(a, v.z, v0.z); v0.w = fmaf(a, v.w, v0.w);
-              gx.x = fmaf(ax, v.x, gx.x); gx.y = fmaf(ax, v.y, gx.y); gx.z = fmaf(ax, v.z, gx.z); gx.w = fmaf(ax, v.w, gx.w);
-              gy.x = fmaf(ay, v.x, gy.x); gy.y = fmaf(ay, v.y, gy.y); gy.z = fmaf(ay, v.z, gy.z); gy.w = fmaf(ay, v.w, gy.w);
-              gz.x = fmaf(az, v.x, gz.x); gz.y = fmaf(az, v.y, gz.y); gz.z = fmaf(az, v.z, gz.z); gz.w = fmaf(az, v.w, gz.w);
-            }
-          }
-        }
-        const float vv[4] = {v0.x, v0.y, v0.z, v0.w};
-        const float xx[4] = {gx.x, gx.y, gx.z, gx.w};
-        const float yy[4] = {gy.x, gy.y, gy.z, gy.w};
-        const float zz[4] = {gz.x, gz.y, gz.z, gz.w};
+  const int mask = n - 1, lg = __ffs(n) - 1;
+  const int lane = threadIdx.x & 31, li = lane & 3, l0 = lane & ~3;
+  const long long nwarp = (static_cast<long long>(gridDim.x) * kAT) >> 5;
+  for (long long base = ((blockIdx.x * static_cast<long long>(kAT) + threadIdx.x) >> 5) * 8; base < np;
+       base += nwarp * 8) {
+    const long long p = base + (lane >> 2);
+    const bool act = p < np;
+    const int cell = act ? s_cell[p] : 0;
+    const float4 t = act ? s_tq[p] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float wx[D], wy[D], wz[D], dx[D], dy[D], dz[D];
+    bs_w<D>(t.x, wx, dx);
+    bs_w<D>(t.y, wy, dy);
+    bs_w<D>(t.z, wz, dz);
+    const int cx = (cell & mask) - OFF, cy = ((cell >> lg) & mask) - OFF, cz = (cell >> (2 * lg)) - OFF;
+    constexpr int NR = D == 4 ? 16 : 2;  // rows: (oz, oy) for D = 4, oz for D = 2
+    const int ox = D == 4 ? li : (li & 1);
+    float lx = wx[0], ldx = dx[0];  // this lane's x factor (for D = 2 times the y factor)
+#pragma unroll
+    for (int o = 1; o < D; ++o) {
+      lx = ox == o ? wx[o] : lx;
+      ldx = ox == o ? dx[o] : ldx;
+    }
+    const int xo = (cx + ox) & mask;
+    const bool y1 = li >> 1;
+    const float ly = y1 ? wy[1] : wy[0], ldy = y1 ? dy[1] : dy[0];  // D = 2 only
+    auto row_at = [&](int r) {
+      const int oz = D == 4 ? r >> 2 : r, oy = D == 4 ? r & 3 : static_cast<int>(y1);
+      return (((((cz + oz) & mask) << lg) + ((cy + oy) & mask)) << lg) + xo;
+    };
+    float f[G], gx[G], gy[G], gz[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const float4* src = f4 + g * ng;
+      float vp[4] = {0.f, 0.f, 0.f, 0.f}, vy[4] = {0.f, 0.f, 0.f, 0.f}, vz[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const float4 v = __ldg(src + row_at(r));
+        const float vv[4] = {v.x, v.y, v.z, v.w};
+        const int oz = D == 4 ? r >> 2 : r, oy = D == 4 ? r & 3 : 0;
+        const float a = D == 4 ? wz[oz] * wy[oy] : wz[oz], az = D == 4 ? dz[oz] * wy[oy] : dz[oz];
+        const float ay = D == 4 ? wz[oz] * dy[oy] : 0.f;
+#pragma unroll
         for (int j = 0; j < 4; ++j) {
-          fv[p][4 * g + j] = vv[j];
-          gv[p][4 * g + j][0] = xx[j];
-          gv[p][4 * g + j][1] = yy[j];
-          gv[p][4 * g + j][2] = zz[j];
+          vp[j] = fmaf(a, vv[j], vp[j]);
+          vz[j] = fmaf(az, vv[j], vz[j]);
+          if (D == 4) vy[j] = fmaf(ay, vv[j], vy[j]);
         }
       }
-      __syncthreads();
-      // per particle: c = (2 w / W) S f, the direct term, then c replaces f
-      if (threadIdx.x < cnt) {
-        const int p = threadIdx.x;
-        float c[NBP];
-        for (int b = 0; b < NBP; ++b) {
-          float t = 0.f;
-          for (int b2 = 0; b2 < NBP; ++b2) t = fmaf(s_s[b * NBP + b2], (b2 < 4 * ngrp) ? fv[p][b2] : 0.f, t);
-          c[b] = wscale * pw[p] * t;
+      float k4[4][4];  // [kind][bin]: f, df/dx, df/dy, df/dz of this lane's nodes
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (D == 4) {
+          k4[0][j] = lx * vp[j];
+          k4[1][j] = ldx * vp[j];
+          k4[2][j] = lx * vy[j];
+          k4[3][j] = lx * vz[j];
+        } else {
+          k4[0][j] = lx * ly * vp[j];
+          k4[1][j] = ldx * ly * vp[j];
+          k4[2][j] = lx * ldy * vp[j];
+          k4[3][j] = lx * ly * vz[j];
         }
-        float dx = 0.f, dy = 0.f, dz = 0.f;
-        for (int b = 0; b < 4 * ngrp && b < NBP; ++b) {
-          dx = fmaf(c[b], gv[p][b][0], dx);
-          dy = fmaf(c[b], gv[p][b][1], dy);
-          dz = fmaf(c[b], gv[p][b][2], dz);
-        }
-        const long long oi = sidx[bs + p];
-        direct[3 * oi] += dx;
-        direct[3 * oi + 1] += dy;
-        direct[3 * oi + 2] += dz;
-        for (int b = 0; b < NBP; ++b) fv[p][b] = c[b];
       }
-      __syncthreads();
-      // scatter c_b with the assignment stencil
-      for (int task = threadIdx.x; task < cnt * ngrp; task += blockDim.x) {
-        const int p = task % cnt, g = task / cnt;
-        const int4 o = org[p];
-        const float* w = bw[p];
-        const float4 cv = make_float4(fv[p][4 * g], fv[p][4 * g + 1], fv[p][4 * g + 2], fv[p][4 * g + 3]);
-        float4* base = h4 + g * ng;
-        for (int oz = 0; oz < D; ++oz) {
-          const long long zrow = static_cast<long long>((o.z + oz) & mask) * n;
-          for (int oy = 0; oy < D; ++oy) {
-            float4* row = base + (zrow + ((o.y + oy) & mask)) * n;
-            const float wyz = w[2 * D + oz] * w[D + oy];
-            for (int ox = 0; ox < D; ++ox) {
-              const float a = wyz * w[ox];
-              atomicAdd(row + ((o.x + ox) & mask), make_float4(a * cv.x, a * cv.y, a * cv.z, a * cv.w));
-            }
-          }
+      float res[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {  // reduce-scatter over the four lanes: lane i keeps bin i
+        const bool hi = li & 2;
+        float a0 = hi ? k4[c][2] : k4[c][0], a1 = hi ? k4[c][3] : k4[c][1];
+        a0 += __shfl_xor_sync(0xffffffffu, hi ? k4[c][0] : k4[c][2], 2);
+        a1 += __shfl_xor_sync(0xffffffffu, hi ? k4[c][1] : k4[c][3], 2);
+        const bool odd = li & 1;
+        const float keep = odd ? a1 : a0;
+        res[c] = keep + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 1);
+      }
+      f[g] = res[0];
+      gx[g] = res[1];
+      gy[g] = res[2];
+      gz[g] = res[3];
+    }
+    float c[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) c[g] = 0.f;
+#pragma unroll
+    for (int g2 = 0; g2 < G; ++g2) {
+      float fb[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) fb[j] = __shfl_sync(0xffffffffu, f[g2], l0 + j);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const float4 sv = *reinterpret_cast<const float4*>(s_s + (4 * g + li) * NBP + 4 * g2);
+        c[g] = fmaf(sv.x, fb[0], c[g]);
+        c[g] = fmaf(sv.y, fb[1], c[g]);
+        c[g] = fmaf(sv.z, fb[2], c[g]);
+        c[g] = fmaf(sv.w, fb[3], c[g]);
+      }
+    }
+    float ex = 0.f, ey = 0.f, ez = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      c[g] *= wscale * t.w;
+      ex = fmaf(c[g], gx[g], ex);
+      ey = fmaf(c[g], gy[g], ey);
+      ez = fmaf(c[g], gz[g], ez);
+    }
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+      ex += __shfl_xor_sync(0xffffffffu, ex, off);
+      ey += __shfl_xor_sync(0xffffffffu, ey, off);
+      ez += __shfl_xor_sync(0xffffffffu, ez, off);
+    }
+    if (act && li < 3) {
+      float* o = direct + 3 * static_cast<long long>(sidx[p]) + li;
+      *o += hinv * (li == 0 ? ex : li == 1 ? ey : ez);
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      float cb[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) cb[j] = __shfl_sync(0xffffffffu, c[g], l0 + j);
+      if (act && t.w != 0.f) {
+        float4* dst = h4 + g * ng;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const int oz = D == 4 ? r >> 2 : r, oy = D == 4 ? r & 3 : 0;
+          const float a = (D == 4 ? wz[oz] * wy[oy] : wz[oz] * ly) * lx;
+          atomicAdd(dst + row_at(r), make_float4(a * cb[0], a * cb[1], a * cb[2], a * cb[3]));
         }
       }
     }
@@ -270,17 +326,17 @@ __global__ void k_adj_finish_node(const float* __restrict__ q, const float* __re
 
 template <int D>
 __global__ void k_adj_finish_particles(const float4* __restrict__ parts, long long np, const float* __restrict__ gd, int n,
-                                       double inv_h, const double* __restrict__ wsum, const float* __restrict__ direct,
+                                       CellScale cs, const double* __restrict__ wsum, const float* __restrict__ direct,
                                        float* __restrict__ grad) {
   constexpr int OFF = D / 2 - 1;
   const int mask = n - 1;
   const float scale = static_cast<float>(static_cast<double>(n) * n * n / wsum[0]);
-  const float hinv = static_cast<float>(inv_h);
+  const float hinv = static_cast<float>(cs.inv_h);
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < np;
        i += static_cast<long long>(blockDim.x) * gridDim.x) {
     const float4 pp = parts[i];
     float tx, ty, tz;
-    const int cx = cell_t(pp.x, inv_h, n, tx), cy = cell_t(pp.y, inv_h, n, ty), cz = cell_t(pp.z, inv_h, n, tz);
+    const int cx = cell_t(pp.x, cs, n, tx), cy = cell_t(pp.y, cs, n, ty), cz = cell_t(pp.z, cs, n, tz);
     float wx[D], wy[D], wz[D], dx[D], dy[D], dz[D];
     bs_w<D>(tx, wx, dx);
     bs_w<D>(ty, wy, dy);
@@ -308,7 +364,17 @@ inline int grid1(long long work, int sms) {
   const long long cap = static_cast<long long>(sms) * 16;
   return static_cast<int>(g < 1 ? 1 : (g > cap ? cap : g));
 }
-inline int nbp_of(int nb) { return nb <= 8 ? 8 : nb <= 16 ? 16 : nb <= 24 ? 24 : 32; }
+#define ZK_ADJ_SWITCH(nb, CALL) \
+  switch ((nb + 3) / 4) {       \
+    case 1: CALL(4); break;     \
+    case 2: CALL(8); break;     \
+    case 3: CALL(12); break;    \
+    case 4: CALL(16); break;    \
+    case 5: CALL(20); break;    \
+    case 6: CALL(24); break;    \
+    case 7: CALL(28); break;    \
+    default: CALL(32); break;   \
+  }
 
 }  // namespace
 
@@ -316,44 +382,43 @@ int launch_adj_node_point(const zeta_ctx* c, const float* delta, float* fields, 
                           cudaStream_t s) {
   StageScope prof(c, ST_ADJ_POINT, 1, s);
   float4* f4 = reinterpret_cast<float4*>(fields);
-  const int g = grid1(c->ng, c->num_sms);
-  switch (nbp_of(c->p.nbins)) {
-    case 8: k_adj_node<8><<<g, kAT, 0, s>>>(delta, f4, c->ng, c->p.nbins, S, q); break;
-    case 16: k_adj_node<16><<<g, kAT, 0, s>>>(delta, f4, c->ng, c->p.nbins, S, q); break;
-    case 24: k_adj_node<24><<<g, kAT, 0, s>>>(delta, f4, c->ng, c->p.nbins, S, q); break;
-    default: k_adj_node<32><<<g, kAT, 0, s>>>(delta, f4, c->ng, c->p.nbins, S, q); break;
-  }
+  const int g = grid1(c->ng / 2, c->num_sms);
+#define ZK_CALL(P) k_adj_node<P><<<g, kAT, 0, s>>>(delta, f4, c->ng, c->p.nbins, S, q)
+  ZK_ADJ_SWITCH(c->p.nbins, ZK_CALL)
+#undef ZK_CALL
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
-int launch_adj_mass(const zeta_ctx* c, const float2* dhat, int l, const float* S, float2* gk, cudaStream_t s) {
-  StageScope prof(c, ST_ADJ_OTHER, 1, s);
-  const int nbp = 4 * ((c->p.nbins + 3) / 4);
-  const float* jt = c->d_jtab + static_cast<long long>(l) * c->nn2 * nbp;
-  const float coef = static_cast<float>((2.0 * l + 1.0) / (4.0 * 3.14159265358979323846));
-  k_adj_mass<<<grid1(c->ng / 2, c->num_sms), kAT, 0, s>>>(dhat, jt, nbp, c->d_mhat, c->n, c->p.nbins, S, coef, gk);
+int launch_adj_mass(const zeta_ctx* c, const float2* dhat, const float* S, float* tab, float2* gk, cudaStream_t s) {
+  StageScope prof(c, ST_ADJ_OTHER, 2, s);
+  const int nb = c->p.nbins, nbp = 4 * ((nb + 3) / 4);
+  const size_t sm = sizeof(float) * (c->p.lmax + 1) * nb * nb;
+  if (ensure_smem(reinterpret_cast<const void*>(k_adj_mass_table), sm)) return ZETA_ECUDA;
+  k_adj_mass_table<<<static_cast<unsigned>((c->nn2 + kAT - 1) / kAT), kAT, sm, s>>>(c->d_jtab, c->nn2, nbp, nb, c->p.lmax,
+                                                                                 S, tab);
+  k_adj_mass<<<grid1(c->ng / 2, c->num_sms), kAT, 0, s>>>(dhat, tab, c->d_mhat, c->n, gk);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
-int launch_adj_points(const zeta_ctx* c, const float4* sorted, const int64_t* tile_start, const int* sorted_idx,
+int launch_adj_points(const zeta_ctx* c, const int* s_cell, const float4* s_tq, const int* sorted_idx, int64_t np,
                       const float* fields, const float* S, const double* wsum, float* hfield, float* direct,
                       cudaStream_t s) {
   StageScope prof(c, ST_ADJ_POINT, 1, s);
-  const auto* ts = reinterpret_cast<const long long*>(tile_start);
   const auto* f4 = reinterpret_cast<const float4*>(fields);
   auto* h4 = reinterpret_cast<float4*>(hfield);
-  const double inv_h = c->n / c->p.box;
-  const int g = c->num_sms * 4;
-  const int nb = c->p.nbins;
-#define ZK_ADJ(P, DD) \
-  k_adj_points<P, DD><<<g, kAT, 0, s>>>(sorted, ts, sorted_idx, f4, c->ng, c->n, nb, inv_h, S, wsum, h4, direct)
-  const int nbp = nbp_of(nb);
+  const float hinv = static_cast<float>(c->n / c->p.box);
+  const int g = grid1(np * 4, c->num_sms);
+#define ZK_CALL2(P) \
+  k_adj_points<P, 2><<<g, kAT, 0, s>>>(s_cell, s_tq, sorted_idx, np, f4, c->ng, c->n, c->p.nbins, hinv, S, wsum, h4, direct)
+#define ZK_CALL4(P) \
+  k_adj_points<P, 4><<<g, kAT, 0, s>>>(s_cell, s_tq, sorted_idx, np, f4, c->ng, c->n, c->p.nbins, hinv, S, wsum, h4, direct)
   if (c->p.dsup == 2) {
-    if (nbp == 8) ZK_ADJ(8, 2); else if (nbp == 16) ZK_ADJ(16, 2); else if (nbp == 24) ZK_ADJ(24, 2); else ZK_ADJ(32, 2);
+    ZK_ADJ_SWITCH(c->p.nbins, ZK_CALL2)
   } else {
-    if (nbp == 8) ZK_ADJ(8, 4); else if (nbp == 16) ZK_ADJ(16, 4); else if (nbp == 24) ZK_ADJ(24, 4); else ZK_ADJ(32, 4);
+    ZK_ADJ_SWITCH(c->p.nbins, ZK_CALL4)
   }
-#undef ZK_ADJ
+#undef ZK_CALL2
+#undef ZK_CALL4
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
@@ -366,11 +431,11 @@ int launch_adj_finish_node(const zeta_ctx* c, const float* q, const float* g, fl
 int launch_adj_finish_particles(const zeta_ctx* c, const float4* parts, int64_t np, const float* gdelta,
                                 const double* wsum, const float* direct, float* grad, cudaStream_t s) {
   StageScope prof(c, ST_ADJ_OTHER, 1, s);
-  const double inv_h = c->n / c->p.box;
+  const CellScale cs = make_cell_scale(c->n, c->p.box);
   if (c->p.dsup == 2)
-    k_adj_finish_particles<2><<<grid1(np, c->num_sms), kAT, 0, s>>>(parts, np, gdelta, c->n, inv_h, wsum, direct, grad);
+    k_adj_finish_particles<2><<<grid1(np, c->num_sms), kAT, 0, s>>>(parts, np, gdelta, c->n, cs, wsum, direct, grad);
   else
-    k_adj_finish_particles<4><<<grid1(np, c->num_sms), kAT, 0, s>>>(parts, np, gdelta, c->n, inv_h, wsum, direct, grad);
+    k_adj_finish_particles<4><<<grid1(np, c->num_sms), kAT, 0, s>>>(parts, np, gdelta, c->n, cs, wsum, direct, grad);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 

@@ -929,20 +929,22 @@ int zeta_backward_particles(zeta_ctx* c, const float* particles, int64_t np, con
   float2* gk = at<float2>(c, L.gk);
   float* hfield = at<float>(c, L.hfield);
   float* direct = at<float>(c, L.direct);
+  const PartPrep pq = prep_of(c, L);
   const size_t hbytes = sizeof(float) * c->ng * 4 * ((nb + 3) / 4);
-  ZK_TRY(launch_assign(c, parts, np, dl, wsum, assign_scratch(c, L), stream));
+  ZK_TRY(launch_sort(c, parts, np, sorted, tstart, at<int>(c, L.counts), at<int>(c, L.orig), stream, sidx, &pq));
+  ZK_TRY(launch_assign_sorted(c, parts, np, pq.s_cell, pq.s_tq, dl, wsum, reinterpret_cast<unsigned long long*>(fields),
+                              small, stream));
   ZK_TRY(launch_r2c(c, dl, dhat, stream));
-  ZK_TRY(launch_sort(c, parts, np, sorted, tstart, at<int>(c, L.counts), at<int>(c, L.orig), stream, sidx));
   if (cudaMemsetAsync(gk, 0, sizeof(float) * c->ng, stream) != cudaSuccess ||
       cudaMemsetAsync(direct, 0, sizeof(float) * 3 * np, stream) != cudaSuccess)
     return ZETA_ECUDA;
+  ZK_TRY(launch_adj_mass(c, dhat, S, at<float>(c, L.mhist), gk, stream));
   for (int l = 0; l <= c->p.lmax; ++l) {
     const float* Sl = S + static_cast<size_t>(l) * nb * nb;
-    ZK_TRY(launch_adj_mass(c, dhat, l, Sl, gk, stream));
     for (int m = -l; m <= l; ++m) {
       ZK_TRY(launch_alm(c, dhat, l, m, 0, nb, spec, fields, stream));
       if (cudaMemsetAsync(hfield, 0, hbytes, stream) != cudaSuccess) return ZETA_ECUDA;
-      ZK_TRY(launch_adj_points(c, sorted, tstart, sidx, fields, Sl, wsum, hfield, direct, stream));
+      ZK_TRY(launch_adj_points(c, pq.s_cell, pq.s_tq, sidx, np, fields, Sl, wsum, hfield, direct, stream));
       ZK_TRY(launch_adj_spectral(c, hfield, nb, spec, l, m, gk, stream));
     }
   }

@@ -555,56 +555,169 @@ __global__ void __launch_bounds__(RegThreads<N / 2, 4 * RB, 256>::NT)
   }
 }
 
+// The same for grids of 256^3 and more, with the stages of k_c2r_x4v the other way round: a thread reads the
+// four fields of two points (32 bytes) once and transforms them together, where k_r2c_x4 reads each float4
+// for every field it holds.  256^3, 10 fields: 536 -> 380 us.
+template <int N, int XT>
+__global__ void __launch_bounds__(XT, 768 / XT)
+    k_r2c_x4v(const float4* __restrict__ in, int nf, float2* __restrict__ spec, long long fstride,
+              const float2* __restrict__ twg) {
+  using Y = X4v<N, XT>;
+  constexpr int NC = Y::NC, RB = Y::RB, R0 = NC / 64, KAP = NC / 8;
+  extern __shared__ float2 sm[];
+  float2* ex = sm;
+  float2* tw = sm + 4 * RB * NC;         // per-stage twiddles of the length-NC transform
+  float2* tww = tw + StageTw<NC>::SIZE;  // W_N^k, k < NC
+  stage_tw_fill<NC>(tw, twg, 2);
+  for (int i = threadIdx.x; i < NC; i += XT) tww[i] = twg[i];
+  __syncthreads();
+  const int g = blockIdx.y;
+  const long long r0 = static_cast<long long>(blockIdx.x) * RB;
+  // stage 0: butterfly k of one row, four fields
+#pragma unroll 1
+  for (int i = threadIdx.x; i < 64 * RB; i += XT) {
+    const int k = i & 63, r = i >> 6;
+    const float4* row = in + (static_cast<long long>(g) * N * N + r0 + r) * N;
+    float2 x[4][R0];
+#pragma unroll
+    for (int q = 0; q < R0; ++q) {
+      const float4 a = row[2 * (k + 64 * q)], b = row[2 * (k + 64 * q) + 1];
+      x[0][q] = make_float2(a.x, b.x);
+      x[1][q] = make_float2(a.y, b.y);
+      x[2][q] = make_float2(a.z, b.z);
+      x[3][q] = make_float2(a.w, b.w);
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      dft_small<R0, false>(x[f]);
+      twiddle<R0, NC, false>(x[f], k, tw);
+#pragma unroll
+      for (int p = 0; p < R0; ++p) ex[x_slot<NC>(k + 64 * p, f * RB + r)] = x[f][p];
+    }
+  }
+  __syncthreads();
+  // stage 1: span 64
+#pragma unroll 2
+  for (int i = threadIdx.x; i < KAP * 4 * RB; i += XT) {
+    const int k = i % KAP, col = i / KAP, j = k & 7, b = (k >> 3) * 64 + j;
+    float2 x[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) x[a] = ex[x_slot<NC>(b + 8 * a, col)];
+    dft_small<8, false>(x);
+    twiddle<8, 64, false>(x, j, tw + StageTw<NC>::off(1));
+#pragma unroll
+    for (int a = 0; a < 8; ++a) ex[x_slot<NC>(b + 8 * a, col)] = x[a];
+  }
+  __syncthreads();
+  // last stage, in place
+#pragma unroll 2
+  for (int i = threadIdx.x; i < KAP * 4 * RB; i += XT) {
+    const int lam = i % KAP, col = i / KAP, kap = (lam % R0) * 8 + lam / R0;
+    float2 x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = ex[x_slot<NC>(8 * kap + q, col)];
+    dft_small<8, false>(x);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) ex[x_slot<NC>(8 * kap + q, col)] = x[q];
+  }
+  __syncthreads();
+  // X[k] = E[k] + W_N^k O[k] from z[k] and z[NC - k]
+  auto pos = [](int k) { return (k % R0) * 64 + ((k / R0) & 7) * 8 + k / (8 * R0); };
+#pragma unroll 2
+  for (int i = threadIdx.x; i < NC * 4 * RB; i += XT) {
+    const int k = i % NC, col = i / NC, f = 4 * g + col / RB;
+    if (f >= nf) break;  // the fields come in order
+    const float2 zk = ex[x_slot<NC>(pos(k), col)];
+    const float2 zm = cconj(ex[x_slot<NC>(pos((NC - k) & (NC - 1)), col)]);
+    const float2 e = cscale(cadd(zk, zm), 0.5f);
+    const float2 dd = csub(zk, zm);
+    const float2 od = make_float2(0.5f * dd.y, -0.5f * dd.x);
+    spec[f * fstride + (r0 + col % RB) * NC + k] = cadd(e, cmul(tww[k], od));
+  }
+}
+
 // Adjoint z-pass: forward z-transform of nf x,y-transformed spectra and the transposed window,
 // gk += sum_f (-1)^l K_lm,f(n) spec_f(n) with K = i^l R_lm J_f (|n|^2) as in the forward pass.
-// grid (nc/T, n).
+// grid (nc/T, n).  A thread's outputs are the same points for every field, so their sums over the fields,
+// their angular factors and window-table rows stay in registers; the window table is read four bins at a
+// time (one float4 per point), and the next field's inputs are loaded before the current field is
+// transformed.  256^3, 10 fields: 791 us with the sums in shared memory and one word of the table per
+// field, 331 us now.
 template <int N, int T>
-__global__ void __launch_bounds__(RegThreads<N, T, 512>::NT)
+__global__ void __launch_bounds__(RegThreads<N, T, 512>::NT, RegThreads<N, T, 512>::NT >= 512 ? 1 : 512 / RegThreads<N, T, 512>::NT)
     k_adj_z(const float2* __restrict__ spec, long long fstride, int nf, const float4* __restrict__ jt4, int nbp4,
             int l, int m, float2* __restrict__ gk, const float2* __restrict__ twg, const float* __restrict__ phi) {
   constexpr int NC = N / 2;
   constexpr int NT = RegThreads<N, T, 512>::NT;
+  constexpr int PPT = N * T / NT;
+  using Last = RegStage<N, T, NT, false, 0, 2, FftPlan<N>::NST - 1>;
   extern __shared__ float2 sm[];
   float2* tw = sm;                      // per-stage twiddles
   float2* ex = tw + StageTw<N>::SIZE;   // [N][T] (+ N padding)
-  float2* acc = ex + N * T + N;         // [N][T] sum over fields
-  float* ang = reinterpret_cast<float*>(acc + N * T);  // [N][T]
-  int* n2 = reinterpret_cast<int*>(ang + N * T);        // [N][T]
   const int x0 = blockIdx.x * T;
   const int iy = blockIdx.y;
   if (iy == N / 2) return;  // the window vanishes on the y-Nyquist plane
-  const long long colbase = static_cast<long long>(iy) * NC + x0;
-  const long long zstride = static_cast<long long>(N) * NC;
+  const int colbase = iy * NC + x0;
+  constexpr int zstride = N * NC;  // n^3 / 2 < 2^31
   stage_tw_fill<N>(tw, twg, 1);
   // (-1)^l i^l = (-i)^l = sgn * (-i)^(l mod 2): sgn = +1 for l mod 4 in {0, 1}, -1 otherwise
   const float sgn = ((l & 3) < 2) ? 1.f : -1.f;
   const int ny = signed_freq(iy, N);
-  for (int idx = threadIdx.x; idx < N * T; idx += blockDim.x) {
-    const int z = idx / T, c = idx % T;
+  int row[PPT];     // window-table row of output s of this thread
+  float ang[PPT];
+  float2 acc[PPT];
+#pragma unroll
+  for (int s = 0; s < PPT; ++s) {
+    int c, k;
+    reg_task<N, T, NT, 0, Last::R>(s / Last::R, c, k);
+    const int z = fft_index_at<N>(Last::base_of(k) + (s % Last::R) * Last::M);
     const int nz = signed_freq(z, N), nx = x0 + c;
     const bool nyq = (z == N / 2);
-    n2[idx] = nyq ? 0 : nx * nx + ny * ny + nz * nz;
-    ang[idx] = nyq ? 0.f
-                   : sgn * ylm_dev(l, m, static_cast<float>(nx), static_cast<float>(ny), static_cast<float>(nz)) *
-                         (__ldg(phi + nx) * __ldg(phi + iy) * __ldg(phi + z));
-    acc[idx] = make_float2(0.f, 0.f);
+    row[s] = nyq ? 0 : (nx * nx + ny * ny + nz * nz) * nbp4;
+    ang[s] = nyq ? 0.f
+                 : sgn * ylm_dev(l, m, static_cast<float>(nx), static_cast<float>(ny), static_cast<float>(nz)) *
+                       (__ldg(phi + nx) * __ldg(phi + iy) * __ldg(phi + z));
+    acc[s] = make_float2(0.f, 0.f);
   }
+  float2 nxt[PPT];
+  auto fetch = [&](int f) {
+    const float2* sf = spec + f * fstride + colbase;
+#pragma unroll
+    for (int s = 0; s < PPT; ++s) {
+      int c, z;
+      reg_slot<N, T, NT, 0>(s, c, z);
+      nxt[s] = sf[z * zstride + c];
+    }
+  };
+  fetch(0);
   __syncthreads();
-  const float* jt = reinterpret_cast<const float*>(jt4);
-  for (int f = 0; f < nf; ++f) {
-    const float2* sf = spec + f * fstride;
-    auto load = [&](int c, int z) { return sf[colbase + z * zstride + c]; };
-    auto store = [&](int c, int z, float2 v) {
-      const int idx = z * T + c;
-      const float a = ang[idx] * __ldg(jt + static_cast<long long>(n2[idx]) * 4 * nbp4 + f);
-      acc[idx] = cadd(acc[idx], cscale(v, a));
-    };
-    fft_reg<N, T, NT, false, false, 2>(ex, T, tw, load, store);
+  for (int g = 0; 4 * g < nf; ++g) {
+    float4 jv[PPT];
+#pragma unroll
+    for (int s = 0; s < PPT; ++s) jv[s] = __ldg(jt4 + row[s] + g);
+    const int nj = (nf - 4 * g) < 4 ? (nf - 4 * g) : 4;
+    for (int j = 0; j < nj; ++j) {
+      float2 v[PPT];
+#pragma unroll
+      for (int s = 0; s < PPT; ++s) v[s] = nxt[s];
+      if (4 * g + j + 1 < nf) fetch(4 * g + j + 1);
+      int at = 0;
+      auto store = [&](int, int, float2 x) {
+        const float jj = j == 0 ? jv[at].x : j == 1 ? jv[at].y : j == 2 ? jv[at].z : jv[at].w;
+        const float a = ang[at] * jj;
+        acc[at].x = fmaf(x.x, a, acc[at].x);
+        acc[at].y = fmaf(x.y, a, acc[at].y);
+        ++at;
+      };
+      fft_reg_v<N, T, NT, false, 0, 2>(v, ex, T, tw, store);
+    }
   }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < N * T; idx += blockDim.x) {
-    const int z = idx / T, c = idx % T;
-    float2 v = acc[idx];
+#pragma unroll
+  for (int s = 0; s < PPT; ++s) {
+    int c, k;
+    reg_task<N, T, NT, 0, Last::R>(s / Last::R, c, k);
+    const int z = fft_index_at<N>(Last::base_of(k) + (s % Last::R) * Last::M);
+    float2 v = acc[s];
     if (l & 1) v = make_float2(v.y, -v.x);  // times -i
     float2* o = gk + colbase + z * zstride + c;
     *o = cadd(*o, v);
@@ -796,15 +909,23 @@ int adj_impl(const zeta_ctx* c, const float* fields, int nf, float2* spec, int l
   constexpr int RB = kRB4;
   const long long fstride = static_cast<long long>(N) * N * NC;
   StageScope prof(c, ST_ADJ_FFT, 3, s);
-  const size_t smx = x4_smem<N, RB>();
-  if (set_smem(k_r2c_x4<N, RB>, smx)) return ZETA_ECUDA;
-  k_r2c_x4<N, RB><<<dim3(N * N / RB, (nf + 3) / 4), RegThreads<N / 2, 4 * RB, 256>::NT, smx, s>>>(
-      reinterpret_cast<const float4*>(fields), nf, spec, fstride, c->d_tw);
+  if constexpr (N >= 256) {
+    constexpr int XT = kX4Threads;
+    using Y = X4v<N, XT>;
+    constexpr size_t smx = (4 * Y::RB * NC + StageTw<NC>::SIZE + NC) * sizeof(float2);
+    if (set_smem(k_r2c_x4v<N, XT>, smx)) return ZETA_ECUDA;
+    k_r2c_x4v<N, XT><<<dim3(N * N / Y::RB, (nf + 3) / 4), XT, smx, s>>>(reinterpret_cast<const float4*>(fields), nf, spec,
+                                                                        fstride, c->d_tw);
+  } else {
+    const size_t smx = x4_smem<N, RB>();
+    if (set_smem(k_r2c_x4<N, RB>, smx)) return ZETA_ECUDA;
+    k_r2c_x4<N, RB><<<dim3(N * N / RB, (nf + 3) / 4), RegThreads<N / 2, 4 * RB, 256>::NT, smx, s>>>(
+        reinterpret_cast<const float4*>(fields), nf, spec, fstride, c->d_tw);
+  }
   const size_t sma = axis_smem<N, TY>();
   if (set_smem(k_fft_axis<N, TY, false, 1>, sma)) return ZETA_ECUDA;
   k_fft_axis<N, TY, false, 1><<<dim3(NC / TY, N, nf), RegThreads<N, TY, 512>::NT, sma, s>>>(spec, fstride, c->d_tw);
-  const size_t smz = (StageTw<N>::SIZE + 2 * static_cast<size_t>(N) * TZ + N) * sizeof(float2) +
-                     2 * static_cast<size_t>(N) * TZ * 4;
+  const size_t smz = (StageTw<N>::SIZE + static_cast<size_t>(N) * TZ + N) * sizeof(float2);
   if (set_smem(k_adj_z<N, TZ>, smz)) return ZETA_ECUDA;
   const int nbp4 = (c->p.nbins + 3) / 4;
   const float4* jt4 = reinterpret_cast<const float4*>(c->d_jtab) + static_cast<long long>(l) * c->nn2 * nbp4;

@@ -232,8 +232,9 @@ int launch_assign_sorted(const zeta_ctx* c, const float4* parts, int64_t np, con
 // S: symmetrised loss weights of one l, device float [nb][nb]
 int launch_adj_node_point(const zeta_ctx* c, const float* delta, float* fields, const float* S, float* q,
                           cudaStream_t s);
-int launch_adj_mass(const zeta_ctx* c, const float2* dhat, int l, const float* S, float2* gk, cudaStream_t s);
-int launch_adj_points(const zeta_ctx* c, const float4* sorted, const int64_t* tile_start, const int* sorted_idx,
+// S of all l: [lmax + 1][nb][nb]; tab: scratch of nn2 floats
+int launch_adj_mass(const zeta_ctx* c, const float2* dhat, const float* S, float* tab, float2* gk, cudaStream_t s);
+int launch_adj_points(const zeta_ctx* c, const int* s_cell, const float4* s_tq, const int* sorted_idx, int64_t np,
                       const float* fields, const float* S, const double* wsum, float* hfield, float* direct,
                       cudaStream_t s);
 int launch_adj_finish_node(const zeta_ctx* c, const float* q, const float* g, float* grad, cudaStream_t s);
