@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <utility>
 
 #include "zeta_internal.h"
 
@@ -22,6 +23,25 @@ struct Layout {
   size_t total = 0;
 };
 
+// (l, m) pairs that a measurement takes together.  On small grids every kernel of one pair is a few
+// microseconds of latency on a machine that is mostly idle, so the pairs share launches as long as their
+// spectra and fields stay within 128 MB, an L2's worth (64^3 with 8 bins: 8 pairs; from 128^3 on mostly
+// one).  64^3, 8 bins, l <= 4, all forms: 4236 us pair by pair,
+// 3864 / 3146 / 2596 / 2423 with a limit of 16 / 32 / 64 / 128 MB.
+int lm_batch(const zeta_ctx* c) {
+  const size_t per = sizeof(float) * static_cast<size_t>(c->ng) * (c->p.nbins + 4 * ((c->p.nbins + 3) / 4));
+  const size_t fit = (static_cast<size_t>(128) << 20) / per;
+  const int pairs = (c->p.lmax + 1) * (c->p.lmax + 1);
+  int b = fit < 1 ? 1 : fit > kMaxLm ? kMaxLm : static_cast<int>(fit);
+  return b < pairs ? b : pairs;
+}
+// ... and of those, the pairs whose interpolated rows are held together (64 MB or one pair's rows)
+size_t rows_bytes(const zeta_ctx* c, int64_t np) {
+  const size_t one = particle_rows_bytes(c, np), all = one * lm_batch(c), cap = static_cast<size_t>(64) << 20;
+  const size_t some = all < cap ? all : cap;
+  return some > one ? some : one;  // grows with np, so a workspace for more particles serves fewer
+}
+
 // Workspace regions of the full measurement for np particles (np may be 0); with backward,
 // also the regions of the gradient calls (placed after the forward ones).
 Layout layout(const zeta_ctx* c, int64_t np, bool backward = false, bool ss = false) {
@@ -35,8 +55,9 @@ Layout layout(const zeta_ctx* c, int64_t np, bool backward = false, bool ss = fa
   const size_t g = static_cast<size_t>(c->ng) * sizeof(float);
   L.delta = take(g);
   L.dhat = take(g);
-  L.spectra = take(g * c->p.nbins);                    // plain half spectra of the C2R passes
-  L.fields = take(g * 4 * ((c->p.nbins + 3) / 4));     // bin-interleaved fields; also the assign accumulator
+  const size_t lmb = static_cast<size_t>(lm_batch(c));
+  L.spectra = take(g * c->p.nbins * lmb);              // plain half spectra of the C2R passes
+  L.fields = take(g * 4 * ((c->p.nbins + 3) / 4) * lmb);  // bin-interleaved fields; also the assign accumulator
   L.partials = take(sizeof(double) * kMaxCtas * c->p.nbins * c->p.nbins);
   if (c->p.tophat_primary > 0) L.dprim = take(g);  // the grid forms' smoothed primary vertex
   L.xi_radii = take(sizeof(double) * 4096);          // radii of zeta_xi_radii
@@ -46,7 +67,7 @@ Layout layout(const zeta_ctx* c, int64_t np, bool backward = false, bool ss = fa
   L.tstart = take(sizeof(int64_t) * static_cast<size_t>(c->ntiles + 1));
   L.counts = take(sizeof(int) * static_cast<size_t>(c->ntiles));
   L.orig = take(sizeof(int) * static_cast<size_t>(np));
-  L.pvals = take(particle_rows_bytes(c, np));  // interpolated particle rows of one (l, m)
+  L.pvals = take(rows_bytes(c, np));  // interpolated particle rows of one (l, m), or of a few
   // prepared particle data (cell, offsets, weight): original order (scratch) and sorted order
   L.o_tile = take(sizeof(int) * static_cast<size_t>(np));
   L.o_cell = take(sizeof(int) * static_cast<size_t>(np));
@@ -340,8 +361,8 @@ int zeta_sum_grid(zeta_ctx* c, const float* delta, const float* alm, int form, d
                        : launch_gram_node_tc(c, delta, alm, part, stream));
   else
     ZK_TRY(launch_gram_gamma(c, delta, alm, part, stream));
-  return launch_reduce(c, part, gram_ctas(c, form == ZETA_SUM_NODE ? (tc_gram(c) ? GK_TC : GK_NODE) : GK_GAMMA),
-                       1.0 / static_cast<double>(c->ng), nullptr, gram, stream);
+  return launch_reduce(c, part,
+                       form == ZETA_SUM_NODE ? gram_ctas(c, tc_gram(c) ? GK_TC : GK_NODE) : gamma_ctas(c), 1.0 / static_cast<double>(c->ng), nullptr, gram, stream);
 }
 
 int zeta_sort_particles(zeta_ctx* c, const float* particles, int64_t np, float* sorted, int64_t* tile_start,
@@ -377,7 +398,7 @@ int zeta_mass_term(zeta_ctx* c, const float* delta_hat, int l, double sign, doub
   ZK_TRY(launch_mass_hist(c, reinterpret_cast<const float2*>(delta_hat), hist, stream));
   ZK_TRY(launch_mass(c, hist, l, part, stream));
   const double scale = sign * (2.0 * l + 1.0) / (4.0 * 3.14159265358979323846);
-  return launch_reduce(c, part, gram_ctas(c, GK_MASS), scale, nullptr, gram, stream);
+  return launch_reduce(c, part, mass_ctas(c), scale, nullptr, gram, stream);
 }
 
 }  // extern "C"
@@ -442,37 +463,77 @@ int measure(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
   const size_t nslot = slots ? static_cast<size_t>(lmax + 1) * (lmax + 1) + lmax + 1 : static_cast<size_t>(lmax + 1);
   const size_t per_form = nslot * nb2;
   if (cudaMemsetAsync(zeta, 0, sizeof(double) * per_form * nforms, stream) != cudaSuccess) return ZETA_ECUDA;
-  // output block of form index f for (l, m) (m > l: the uniform term of l)
-  auto out = [&](int f, int l, int m) {
-    size_t slot = l;
-    if (slots) slot = m > l ? static_cast<size_t>(lmax + 1) * (lmax + 1) + l : static_cast<size_t>(l) * l + l + m;
-    return zeta + f * per_form + slot * nb2;
-  };
   const double inv_ng = 1.0 / static_cast<double>(c->ng);
-  for (int l = 0; l <= lmax; ++l) {
-    if (want_p && (l * l) % lm_size == lm_rank) {
-      ZK_TRY(launch_mass(c, hist, l, part, stream));
-      ZK_TRY(launch_reduce(c, part, gram_ctas(c, GK_MASS), -(2.0 * l + 1.0) / (4.0 * 3.14159265358979323846), nullptr,
-                           out(idx_part, l, l + 1), stream, slots));
+  // output slot of (l, m) (m > l: the uniform term of l)
+  auto slot = [&](int l, int m) {
+    return !slots ? l : m > l ? (lmax + 1) * (lmax + 1) + l : l * l + l + m;
+  };
+  // the uniform term of the multipoles this call owns, as many at a time as the partials hold
+  if (want_p) {
+    const int per = mass_ctas(c);
+    for (int l = 0; l <= lmax;) {
+      int nl = 0;
+      while (l + nl <= lmax && nl < kMaxLm && (nl + 1) * per <= kMaxCtas &&
+             ((l + nl) * (l + nl)) % lm_size == lm_rank)
+        ++nl;
+      if (nl == 0) {  // not this call's
+        ++l;
+        continue;
+      }
+      ReduceList r;
+      for (int k = l; k < l + nl; ++k) {
+        r.at[r.n] = slot(k, k + 1);
+        r.scale[r.n++] = -(2.0 * k + 1.0) / (4.0 * 3.14159265358979323846);
+      }
+      ZK_TRY(launch_mass(c, hist, l, part, stream, nl));
+      ZK_TRY(launch_reduce_list(c, part, per, r, nullptr, zeta + idx_part * per_form, stream, slots));
+      l += nl;
     }
-    for (int m = -l; m <= l; ++m) {
-      if ((l * l + l + m) % lm_size != lm_rank) continue;
-      ZK_TRY(launch_alm(c, dhat, l, m, 0, nb, at<float2>(c, L.spectra), fields, stream, bf16f));
-      if (idx_node >= 0) {
-        ZK_TRY(!tc_gram(c) ? launch_gram_node(c, prim, fields, part, stream, bf16f)
-                           : launch_gram_node_tc(c, prim, fields, part, stream));
-        ZK_TRY(launch_reduce(c, part, gram_ctas(c, tc_gram(c) ? GK_TC : GK_NODE), inv_ng, nullptr,
-                             out(idx_node, l, m), stream, slots));
+  }
+  std::vector<std::pair<int, int>> pairs;  // (l, m) of this call, in the order of their sums
+  for (int l = 0; l <= lmax; ++l)
+    for (int m = -l; m <= l; ++m)
+      if ((l * l + l + m) % lm_size == lm_rank) pairs.emplace_back(l, m);
+  const int lmb = lm_batch(c);
+  const size_t field_floats = static_cast<size_t>(c->ng) * 4 * ((nb + 3) / 4) / (bf16f ? 2 : 1);
+  const size_t one_row = want_p ? particle_rows_bytes(c, np) : 1;
+  // runs a form's Gram over the pairs i0 .. i0 + k of the batch and adds the results, k as large as the
+  // partials (parts per pair) and the form allow
+  auto form_sums = [&](const LmList& lms, int parts, int most, int idx, double scale, const double* wdiv, auto gram) -> int {
+    if (most > kMaxCtas / parts) most = kMaxCtas / parts;
+    for (int i0 = 0; i0 < lms.n; i0 += most) {
+      const int k = lms.n - i0 < most ? lms.n - i0 : most;
+      ZK_TRY(gram(fields + i0 * field_floats, k));
+      ReduceList r;
+      for (int i = i0; i < i0 + k; ++i) {
+        r.at[r.n] = slot(lms.l[i], lms.m[i]);
+        r.scale[r.n++] = scale;
       }
-      if (idx_gamma >= 0) {
-        ZK_TRY(launch_gram_gamma(c, prim, fields, part, stream));
-        ZK_TRY(launch_reduce(c, part, gram_ctas(c, GK_GAMMA), inv_ng, nullptr, out(idx_gamma, l, m), stream, slots));
-      }
-      if (idx_part >= 0) {
-        ZK_TRY(launch_gram_particles(c, q.s_cell, q.s_tq, tstart, np, fields, at<float>(c, L.pvals), part, stream));
-        ZK_TRY(launch_reduce(c, part, gram_particle_parts(c), 1.0, wsum, out(idx_part, l, m), stream, slots));
-      }
+      ZK_TRY(launch_reduce_list(c, part, parts, r, wdiv, zeta + idx * per_form, stream, slots));
     }
+    return ZETA_OK;
+  };
+  for (size_t p0 = 0; p0 < pairs.size(); p0 += lmb) {
+    LmList lms;
+    for (size_t i = p0; i < pairs.size() && i < p0 + lmb; ++i) lms.add(pairs[i].first, pairs[i].second);
+    ZK_TRY(launch_alm_list(c, dhat, lms, 0, nb, at<float2>(c, L.spectra), fields, stream, bf16f));
+    if (idx_node >= 0) {
+      if (tc_gram(c))  // the tensor-core Grams take one pair at a time
+        ZK_TRY(form_sums(lms, gram_ctas(c, GK_TC), 1, idx_node, inv_ng, nullptr,
+                         [&](const float* f, int) { return launch_gram_node_tc(c, prim, f, part, stream); }));
+      else
+        ZK_TRY(form_sums(lms, gram_ctas(c, GK_NODE), kMaxLm, idx_node, inv_ng, nullptr,
+                         [&](const float* f, int k) { return launch_gram_node(c, prim, f, part, stream, bf16f, k); }));
+    }
+    if (idx_gamma >= 0)
+      ZK_TRY(form_sums(lms, gamma_ctas(c), kMaxLm, idx_gamma, inv_ng, nullptr,
+                       [&](const float* f, int k) { return launch_gram_gamma(c, prim, f, part, stream, k); }));
+    if (idx_part >= 0)
+      ZK_TRY(form_sums(lms, gram_particle_parts(c), static_cast<int>(rows_bytes(c, np) / one_row), idx_part, 1.0, wsum,
+                       [&](const float* f, int k) {
+                         return launch_gram_particles(c, q.s_cell, q.s_tq, tstart, np, f, at<float>(c, L.pvals), part,
+                                                      stream, k);
+                       }));
   }
   return ZETA_OK;
 }

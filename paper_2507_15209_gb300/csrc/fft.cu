@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256) k_c2r_x(float2* __restrict__ data, long l
 // The half-length complex transform takes Z[k] = (X[k] + conj X[NC-k]) + i e^{2 pi i k/N}
 // (X[k] - conj X[NC-k]) (X[NC] = 0) straight from global memory; its outputs z[j] =
 // (x[2j], x[2j+1]) are gathered in shared memory and leave as float4 bin groups.
-// grid (n*n/RB, ngroups); spec holds nf plain half spectra, fstride complex apart.
+// grid (n*n/RB, ngroups, (l, m) pairs); spec holds nf plain half spectra per pair, fstride complex apart.
 template <int N, int RB, bool BF16 = false>
 __global__ void __launch_bounds__(RegThreads<N / 2, 4 * RB, 256>::NT)
     k_c2r_x4(const float2* __restrict__ spec, long long fstride, int nf, float4* __restrict__ out,
@@ -181,6 +181,7 @@ __global__ void __launch_bounds__(RegThreads<N / 2, 4 * RB, 256>::NT)
   float2* ex = tw2 + StageTw<NC>::SIZE;  // [NC][PS] exchange, then the outputs in natural order
   float2* res = ex;
   const int g = blockIdx.y;
+  spec += blockIdx.z * nf * fstride;  // blockIdx.z: (l, m) pair; their fields follow each other
   const long long r0 = static_cast<long long>(blockIdx.x) * RB;
   for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twg[i];
   stage_tw_fill<NC>(tw2, twg, 2);
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(RegThreads<N / 2, 4 * RB, 256>::NT)
     const int r = idx / NC, j = idx % NC;
     const float2* src = res + j * PS + r;
     const float2 z0 = src[0], z1 = src[RB], z2 = src[2 * RB], z3 = src[3 * RB];
-    const long long at = (static_cast<long long>(g) * N * N + r0 + r) * N + 2 * j;
+    const long long at = (static_cast<long long>(blockIdx.z * gridDim.y + g) * N * N + r0 + r) * N + 2 * j;
     if constexpr (BF16) {  // four bins of a point as bfloat16 (8 bytes), rounded to nearest even
       uint4 v;
       v.x = bf16x2(z0.x, z1.x);
@@ -426,11 +427,26 @@ struct AlmZ {
   }
 };
 
-template <int N, int T>
+// MULTI (small grids): blockIdx.z = (l, m) of the list times chunk of fpc fields; the fields of the list's
+// pairs follow each other in out.  A 64^3 grid has 132 CTAs of two warps, each transforming its rows
+// for every field in turn (25 us); with one launch for eight pairs and two fields per CTA the machine
+// is full.
+template <int N, int T, bool MULTI>
 __global__ void __launch_bounds__(AlmZ<N, T>::NT, AlmZ<N, T>::MINB)
-    k_alm_z(const float2* __restrict__ dhat, float2* __restrict__ out, long long fstride, int nf,
-            const float4* __restrict__ jt4, int nbp4, int l, int m, const float2* __restrict__ twg,
-            const float* __restrict__ phi) {
+    k_alm_z(const float2* __restrict__ dhat, float2* __restrict__ out, long long fstride, int nfields,
+            const float4* __restrict__ jt4, int nbp4, LmList lms, long long jstride, int fpc,
+            const float2* __restrict__ twg, const float* __restrict__ phi) {
+  int f0 = 0, nf = nfields, l = lms.l[0], m = lms.m[0];
+  if constexpr (MULTI) {
+    const int nch = (nfields + fpc - 1) / fpc;
+    const int lm = blockIdx.z / nch;
+    f0 = (blockIdx.z % nch) * fpc;
+    nf = f0 + fpc < nfields ? f0 + fpc : nfields;
+    l = lms.l[lm];
+    m = lms.m[lm];
+    out += lm * nfields * fstride;
+    jt4 += l * jstride;
+  }
   constexpr int NC = N / 2;
   constexpr int NT = AlmZ<N, T>::NT;
   constexpr int PPT = AlmZ<N, T>::PPT;
@@ -448,7 +464,7 @@ __global__ void __launch_bounds__(AlmZ<N, T>::NT, AlmZ<N, T>::MINB)
   const int colbase[2] = {iy * NC + x0, iy2 * NC + x0};
   constexpr int zstride = N * NC;
   if (iy == N / 2) {  // y-Nyquist row: the window is zero
-    for (int f = 0; f < nf; ++f)
+    for (int f = f0; f < nf; ++f)
       for (int idx = threadIdx.x; idx < N * T; idx += blockDim.x) {
         const int z = idx / T, c = idx % T;
         out[f * fstride + colbase[0] + z * zstride + c] = make_float2(0.f, 0.f);
@@ -479,10 +495,10 @@ __global__ void __launch_bounds__(AlmZ<N, T>::NT, AlmZ<N, T>::MINB)
                                  (pxz * __ldg(phi + iy2));
       pd[(PPT + s) * NT + threadIdx.x] = cscale(dhat[colbase[1] + z * zstride + c], a2);
     }
-    jn[s] = __ldg(jt4 + row);
+    jn[s] = __ldg(jt4 + row + (f0 >> 2));
   }
   __syncthreads();
-  for (int g = 0; 4 * g < nf; ++g) {
+  for (int g = f0 >> 2; 4 * g < nf; ++g) {
     float4 jv[PPT];
 #pragma unroll
     for (int s = 0; s < PPT; ++s) jv[s] = jn[s];
@@ -491,7 +507,7 @@ __global__ void __launch_bounds__(AlmZ<N, T>::NT, AlmZ<N, T>::MINB)
       for (int s = 0; s < PPT; ++s) jn[s] = __ldg(jt4 + pn[s * NT + threadIdx.x] + g + 1);
     }
     const int nj = (nf - 4 * g) < 4 ? (nf - 4 * g) : 4;
-    for (int j = 0; j < nj; ++j) {
+    for (int j = MULTI ? f0 & 3 : 0; j < nj; ++j) {
       const int f = 4 * g + j;
       for (int r = 0; r < nrow; ++r) {
         float2 v[PPT];
@@ -788,16 +804,38 @@ int c2r_impl(const zeta_ctx* c, float2* data, int nf, cudaStream_t s, bool do_y)
 // alm_shape, chosen by zeta_autotune; 0 is the default): z-pass columns T (8 or 4), y-pass
 // columns TY (16 or 8), x-pass rows RB (4 or 2).
 template <int N, int T>
-int alm_z_pass(const zeta_ctx* c, const float2* dhat, int l, int b0, int m, int nf, float2* spec, cudaStream_t s) {
+int alm_z_pass(const zeta_ctx* c, const float2* dhat, const LmList& lms, int b0, int nf, float2* spec, cudaStream_t s) {
   constexpr int NC = N / 2;
   const long long fstride = static_cast<long long>(N) * N * NC;
   StageScope prof(c, ST_ALM_Z, 1, s);
   const size_t smz = AlmZ<N, T>::smem();
-  if (set_smem(k_alm_z<N, T>, smz)) return ZETA_ECUDA;
   const int nbp4 = (c->p.nbins + 3) / 4;
-  const float4* jt4 = reinterpret_cast<const float4*>(c->d_jtab) + static_cast<long long>(l) * c->nn2 * nbp4 + b0 / 4;
-  k_alm_z<N, T><<<dim3(NC / T, N / 2 + 1), AlmZ<N, T>::NT, smz, s>>>(dhat, spec, fstride, nf, jt4, nbp4, l, m,
-                                                                      c->d_tw, c->d_phi);
+  const float4* jt4 = reinterpret_cast<const float4*>(c->d_jtab) + b0 / 4;
+  const long long jstride = c->nn2 * nbp4;
+  if constexpr (N <= 128) {
+    // fields per CTA: all of them, unless that leaves SMs without a CTA and the fields are few; then four,
+    // two or one, until there are two CTAs per SM.  The angular factors are formed once more per chunk.
+    // us in one chunk / split: 64^3 (132 CTAs) 8 fields 25 / 18, 9 fields 33 / 29 (all three passes), 13
+    // fields 37 / 41, 20 fields 45 / 47; 128^3 (520 CTAs) 13 fields 55 / 77.
+    const long long ctas = static_cast<long long>(NC / T) * (N / 2 + 1) * lms.n;
+    int fpc = nf;
+    if (ctas < c->num_sms && nf <= 12)
+      for (int t = 4; t >= 1 && ctas * ((nf + fpc - 1) / fpc) < 2 * c->num_sms; t /= 2)
+        if (t < nf) fpc = t;
+    if (lms.n > 1 || fpc < nf) {
+      if (set_smem(k_alm_z<N, T, true>, smz)) return ZETA_ECUDA;
+      k_alm_z<N, T, true><<<dim3(NC / T, N / 2 + 1, lms.n * ((nf + fpc - 1) / fpc)), AlmZ<N, T>::NT, smz, s>>>(
+          dhat, spec, fstride, nf, jt4, nbp4, lms, jstride, fpc, c->d_tw, c->d_phi);
+      return check_launch();
+    }
+  }
+  if (set_smem(k_alm_z<N, T, false>, smz)) return ZETA_ECUDA;
+  for (int i = 0; i < lms.n; ++i) {
+    LmList one;
+    one.add(lms.l[i], lms.m[i]);
+    k_alm_z<N, T, false><<<dim3(NC / T, N / 2 + 1), AlmZ<N, T>::NT, smz, s>>>(
+        dhat, spec + i * nf * fstride, fstride, nf, jt4 + lms.l[i] * jstride, nbp4, one, jstride, nf, c->d_tw, c->d_phi);
+  }
   return check_launch();
 }
 
@@ -813,7 +851,7 @@ int alm_y_pass(const zeta_ctx* c, int nf, float2* spec, cudaStream_t s) {
 }
 
 template <int N, int RB>
-int alm_x_pass(const zeta_ctx* c, int nf, const float2* spec, float* out, cudaStream_t s, bool bf16) {
+int alm_x_pass(const zeta_ctx* c, int nlm, int nf, const float2* spec, float* out, cudaStream_t s, bool bf16) {
   constexpr int NC = N / 2;
   const long long fstride = static_cast<long long>(N) * N * NC;
   StageScope prof(c, ST_ALM_X, 1, s);
@@ -825,40 +863,39 @@ int alm_x_pass(const zeta_ctx* c, int nf, const float2* spec, float* out, cudaSt
       constexpr int XT = kX4Threads;
       using Y = X4v<N, XT>;
       const dim3 grid(N * N / Y::RB, ng4);
-      if (bf16) {
-        if (set_smem(k_c2r_x4v<N, XT, true>, Y::SMEM)) return ZETA_ECUDA;
-        k_c2r_x4v<N, XT, true><<<grid, XT, Y::SMEM, s>>>(spec, fstride, nf, out, c->d_tw);
-      } else {
-        if (set_smem(k_c2r_x4v<N, XT, false>, Y::SMEM)) return ZETA_ECUDA;
-        k_c2r_x4v<N, XT, false><<<grid, XT, Y::SMEM, s>>>(spec, fstride, nf, out, c->d_tw);
-      }
+      const size_t per = static_cast<size_t>(ng4) * N * N * N * (bf16 ? 2 : 4);  // floats of one pair's fields
+      if (set_smem(bf16 ? k_c2r_x4v<N, XT, true> : k_c2r_x4v<N, XT, false>, Y::SMEM)) return ZETA_ECUDA;
+      for (int i = 0; i < nlm; ++i)
+        (bf16 ? k_c2r_x4v<N, XT, true> : k_c2r_x4v<N, XT, false>)<<<grid, XT, Y::SMEM, s>>>(
+            spec + i * nf * fstride, fstride, nf, out + i * per, c->d_tw);
       return check_launch();
     }
   }
   if (bf16) {
     if (set_smem(k_c2r_x4<N, RB, true>, smx)) return ZETA_ECUDA;
-    k_c2r_x4<N, RB, true><<<dim3(N * N / RB, ng4), RegThreads<N / 2, 4 * RB, 256>::NT, smx, s>>>(
+    k_c2r_x4<N, RB, true><<<dim3(N * N / RB, ng4, nlm), RegThreads<N / 2, 4 * RB, 256>::NT, smx, s>>>(
         spec, fstride, nf, reinterpret_cast<float4*>(out), c->d_tw);
   } else {
     if (set_smem(k_c2r_x4<N, RB>, smx)) return ZETA_ECUDA;
-    k_c2r_x4<N, RB><<<dim3(N * N / RB, ng4), RegThreads<N / 2, 4 * RB, 256>::NT, smx, s>>>(
+    k_c2r_x4<N, RB><<<dim3(N * N / RB, ng4, nlm), RegThreads<N / 2, 4 * RB, 256>::NT, smx, s>>>(
         spec, fstride, nf, reinterpret_cast<float4*>(out), c->d_tw);
   }
   return check_launch();
 }
 
 template <int N>
-int alm_impl(const zeta_ctx* c, const float2* dhat, int l, int m, int b0, int nf, float2* spec, float* out,
+int alm_impl(const zeta_ctx* c, const float2* dhat, const LmList& lms, int b0, int nf, float2* spec, float* out,
              cudaStream_t s, bool bf16) {
   constexpr int NC = N / 2;
   constexpr int T0 = kTz < NC ? kTz : NC, T1 = 4 < NC ? 4 : NC;
   constexpr int Y0 = kTy < NC ? kTy : NC, Y1 = 8 < NC ? 8 : NC;
-  int rc = c->alm_shape[0] ? alm_z_pass<N, T1>(c, dhat, l, b0, m, nf, spec, s)
-                           : alm_z_pass<N, T0>(c, dhat, l, b0, m, nf, spec, s);
+  int rc = c->alm_shape[0] ? alm_z_pass<N, T1>(c, dhat, lms, b0, nf, spec, s)
+                           : alm_z_pass<N, T0>(c, dhat, lms, b0, nf, spec, s);
   if (rc != ZETA_OK) return rc;
-  rc = c->alm_shape[1] ? alm_y_pass<N, Y1>(c, nf, spec, s) : alm_y_pass<N, Y0>(c, nf, spec, s);
+  rc = c->alm_shape[1] ? alm_y_pass<N, Y1>(c, lms.n * nf, spec, s) : alm_y_pass<N, Y0>(c, lms.n * nf, spec, s);
   if (rc != ZETA_OK) return rc;
-  return c->alm_shape[2] ? alm_x_pass<N, 2>(c, nf, spec, out, s, bf16) : alm_x_pass<N, kRB4>(c, nf, spec, out, s, bf16);
+  return c->alm_shape[2] ? alm_x_pass<N, 2>(c, lms.n, nf, spec, out, s, bf16)
+                         : alm_x_pass<N, kRB4>(c, lms.n, nf, spec, out, s, bf16);
 }
 
 // Full inverse of nf half spectra in place: z-, y- and x-passes.
@@ -894,11 +931,18 @@ int launch_r2c(const zeta_ctx* c, const float* delta, float2* dhat, cudaStream_t
 #undef ZK_CALL
 }
 
-int launch_alm(const zeta_ctx* c, const float2* dhat, int l, int m, int b0, int nf, float2* spec, float* out,
-               cudaStream_t s, bool bf16) {
-#define ZK_CALL(NN) alm_impl<NN>(c, dhat, l, m, b0, nf, spec, out, s, bf16)
+int launch_alm_list(const zeta_ctx* c, const float2* dhat, const LmList& lms, int b0, int nf, float2* spec, float* out,
+                    cudaStream_t s, bool bf16) {
+#define ZK_CALL(NN) alm_impl<NN>(c, dhat, lms, b0, nf, spec, out, s, bf16)
   ZK_DISPATCH_N(c->n, ZK_CALL)
 #undef ZK_CALL
+}
+
+int launch_alm(const zeta_ctx* c, const float2* dhat, int l, int m, int b0, int nf, float2* spec, float* out,
+               cudaStream_t s, bool bf16) {
+  LmList one;
+  one.add(l, m);
+  return launch_alm_list(c, dhat, one, b0, nf, spec, out, s, bf16);
 }
 
 template <int N>

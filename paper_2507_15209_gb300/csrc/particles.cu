@@ -42,6 +42,7 @@ struct TileWalk {
   const long long* ts;
   long long ntiles;
   int nt;
+  __device__ __forceinline__ long long count() const { return ts[ntiles]; }  // particles
   __device__ __forceinline__ bool tile(long long k, long long& s0, long long& s1, int& tx, int& ty, int& tz) const {
     const long long i = blockIdx.x + k * gridDim.x;
     if (i >= ntiles) return false;
@@ -204,6 +205,10 @@ __global__ void __launch_bounds__(kIThreads, 3)
   const TileWalk walk{tile_start, static_cast<long long>(nt) * nt * nt, nt};
   constexpr int OFF = D / 2 - 1;
   const int mask = n - 1;
+  if (blockIdx.y) {  // (l, m) pair
+    f4 += static_cast<long long>(blockIdx.y) * ngrp * ng;
+    pvals += static_cast<long long>(blockIdx.y) * walk.count() * NBP;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kKS; ++s) {
@@ -428,6 +433,10 @@ __global__ void __launch_bounds__(kThreadsL1, 1)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int NW = kThreadsL1 / 32;
   // lane -> (particle slot, bin group, x offset)
+  if (blockIdx.y) {  // (l, m) pair
+    f4 += static_cast<long long>(blockIdx.y) * ngrp * ng;
+    pvals += static_cast<long long>(blockIdx.y) * walk.count() * NBP;
+  }
   const int LP = D * ngrp, PPW = 32 / LP;
   const int ps = lane / LP, q = (lane % LP) / D, ox = lane % D;
   const bool lane_on = ps < PPW;
@@ -531,6 +540,8 @@ __global__ void __launch_bounds__(kThreads) k_gram_rows(const float* __restrict_
   using G = Gram<NBP>;
   constexpr int GV = NBP / 4;
   extern __shared__ __align__(16) unsigned char smraw[];
+  pvals += static_cast<long long>(blockIdx.y) * np * NBP;  // blockIdx.y: (l, m) pair
+  partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
   float* vals = reinterpret_cast<float*>(smraw);
   float* wts = vals + kPB * G::NBS;
   double* red = reinterpret_cast<double*>(smraw);  // reused after the main loop
@@ -587,29 +598,29 @@ constexpr int kRowsCtasPerSm = 2;
 
 template <int NBP, int D>
 int part_impl(const zeta_ctx* c, const int* s_cell, const float4* s_tq, const int64_t* tile_start, int64_t np,
-              const float* alm, float* pvals, double* partials, cudaStream_t s) {
+              const float* alm, float* pvals, double* partials, cudaStream_t s, int nlm) {
   StageScope prof(c, ST_GRAM_PART, part_staged_on(c) + part_l1_on(c) + 1, s);
   const long long* ts = reinterpret_cast<const long long*>(tile_start);
   const float4* f4 = reinterpret_cast<const float4*>(alm);
   if (part_staged_on(c)) {
     const size_t sm = InterpSmem<NBP, D>::BYTES;
     if (prep(k_interp_part<NBP, D>, sm)) return ZETA_ECUDA;
-    k_interp_part<NBP, D><<<gram_ctas(c, GK_PART), kIThreads, sm, s>>>(s_cell, s_tq, ts, f4, c->ng, c->n,
+    k_interp_part<NBP, D><<<dim3(gram_ctas(c, GK_PART), nlm), kIThreads, sm, s>>>(s_cell, s_tq, ts, f4, c->ng, c->n,
                                                                        c->p.nbins, c->staged_min, c->d_daub, pvals,
                                                                        c->d_status);
   }
   if (part_l1_on(c)) {
     const size_t sm = InterpL1Smem<NBP, D>::BYTES;
     if (prep(k_interp_part_l1<NBP, D>, sm)) return ZETA_ECUDA;
-    k_interp_part_l1<NBP, D><<<c->num_sms, kThreadsL1, sm, s>>>(s_cell, s_tq, ts, f4, c->ng, c->n, c->p.nbins,
+    k_interp_part_l1<NBP, D><<<dim3(c->num_sms, nlm), kThreadsL1, sm, s>>>(s_cell, s_tq, ts, f4, c->ng, c->n, c->p.nbins,
                                                                 c->staged_min, c->d_daub, pvals);
   }
   if constexpr (NBP <= 20) {  // register-blocked Gram of the rows (sums.cu), one CTA per SM
-    return launch_gram_rows_rb(c, pvals, s_tq, np, partials, gram_particle_parts(c), s);
+    return launch_gram_rows_rb(c, pvals, s_tq, np, partials, gram_particle_parts(c), s, nlm);
   }
   const size_t sm = smem_rows<NBP>();
   if (prep(k_gram_rows<NBP>, sm)) return ZETA_ECUDA;
-  k_gram_rows<NBP><<<gram_particle_parts(c), kThreads, sm, s>>>(pvals, s_tq, np, c->p.nbins, partials);
+  k_gram_rows<NBP><<<dim3(gram_particle_parts(c), nlm), kThreads, sm, s>>>(pvals, s_tq, np, c->p.nbins, partials);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
@@ -708,13 +719,13 @@ size_t particle_rows_bytes(const zeta_ctx* c, int64_t np) {
 }
 
 int launch_gram_particles(const zeta_ctx* c, const int* s_cell, const float4* s_tq, const int64_t* tile_start,
-                          int64_t np, const float* alm, float* pvals, double* partials, cudaStream_t s) {
+                          int64_t np, const float* alm, float* pvals, double* partials, cudaStream_t s, int nlm) {
   if (c->p.dsup == 2) {
-#define ZK_CALL(P) part_impl<P, 2>(c, s_cell, s_tq, tile_start, np, alm, pvals, partials, s)
+#define ZK_CALL(P) part_impl<P, 2>(c, s_cell, s_tq, tile_start, np, alm, pvals, partials, s, nlm)
     ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
   } else {
-#define ZK_CALL(P) part_impl<P, 4>(c, s_cell, s_tq, tile_start, np, alm, pvals, partials, s)
+#define ZK_CALL(P) part_impl<P, 4>(c, s_cell, s_tq, tile_start, np, alm, pvals, partials, s, nlm)
     ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
   }

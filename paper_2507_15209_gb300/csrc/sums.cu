@@ -44,6 +44,8 @@ __global__ void __launch_bounds__(kThreads) k_gram_node(const float* __restrict_
   using G = Gram<NBP, kNodeCons>;
   using R = NodeRing<NBP>;
   extern __shared__ __align__(16) unsigned char smraw[];
+  f4 += static_cast<long long>(blockIdx.y) * ((nb + 3) / 4) * ng;  // blockIdx.y: (l, m) pair
+  partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
   float* ring = reinterpret_cast<float*>(smraw);
   unsigned long long* full = reinterpret_cast<unsigned long long*>(smraw + kNKS * R::SLOTF * sizeof(float));
   unsigned long long* empty = full + kNKS;
@@ -297,6 +299,9 @@ __global__ void __launch_bounds__(kRbThreads, 1)
   using T = Tri<NBP>;
   using Lo = RbLayout<NBP, MODE>;
   extern __shared__ __align__(128) unsigned char smq[];
+  // blockIdx.y: (l, m) pair; its fields or rows hold 4 NBP (bfloat16: 2 NBP) bytes a point
+  fields += static_cast<long long>(blockIdx.y) * ng * NBP * (MODE == 1 ? 2 : 4);
+  partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
   unsigned char* ring = smq;                                                               // [kRbSlots][SLOT]
   unsigned long long* full = reinterpret_cast<unsigned long long*>(smq + kRbSlots * Lo::SLOT);
   unsigned long long* empty = full + kRbSlots;
@@ -427,6 +432,8 @@ __global__ void __launch_bounds__(kThreads)
   using S = GammaShape<NBP, D>;
   constexpr int K = S::K, NC = S::NC, OFF = S::OFF;
   extern __shared__ __align__(16) unsigned char smraw[];
+  f4 += static_cast<long long>(blockIdx.y) * ((nb + 3) / 4) * ng;  // blockIdx.y: (l, m) pair
+  partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
   float* vals = reinterpret_cast<float*>(smraw);             // [kPB][NBS]
   float* wts = vals + kPB * G::NBS;                           // [kPB]
   float4* xbuf = reinterpret_cast<float4*>(smraw);           // [ch][cell][oz][oy][kx], aliases vals
@@ -631,6 +638,8 @@ __global__ void __launch_bounds__(kThreads) k_gram_mass(const unsigned long long
                                                         double* __restrict__ partials) {
   using G = Gram<NBP>;
   extern __shared__ __align__(16) unsigned char smraw[];
+  jt += blockIdx.y * nn2 * (4 * ((nb + 3) / 4));  // blockIdx.y: multipole, from the first one's table on
+  partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
   float* vals = reinterpret_cast<float*>(smraw);
   float* wts = vals + kPB * G::NBS;
   double* red = reinterpret_cast<double*>(smraw);  // reused after the main loop
@@ -678,6 +687,42 @@ __global__ void k_reduce(const double* __restrict__ part, int nparts, int nb, do
     // in a slot and added later (zeta_reduce_lm) rounds exactly as one added here
     const double c = __dmul_rn(sc, sum);
     out[e] = store ? c : __dadd_rn(out[e], c);
+  }
+}
+
+// Several contributions: one CTA per output entry, warp i sums contribution i's partials like k_reduce, then
+// thread 0 adds the products in the order of the list, so the result is that of k_reduce called in turn.
+__global__ void k_reduce_list(const double* __restrict__ part, int nparts, int nb, ReduceList list,
+                              const double* __restrict__ wdiv, double* __restrict__ out, int store) {
+  __shared__ double prod[kMaxLm];
+  const int e = blockIdx.x, i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = e / nb, c = e % nb;
+  const int lo = r < c ? r : c, hi = r < c ? c : r;
+  const double* p = part + static_cast<long long>(i) * nparts * nb * nb + lo * nb + hi;
+  double sum = 0.0;
+#pragma unroll 4
+  for (int k = lane; k < nparts; k += 32) sum += p[static_cast<long long>(k) * nb * nb];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  if (lane == 0) {
+    double sc = list.scale[i];
+    if (wdiv) sc /= *wdiv;
+    prod[i] = __dmul_rn(sc, sum);
+    if (store) out[static_cast<long long>(list.at[i]) * nb * nb + e] = prod[i];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && !store) {
+    int at = -1;
+    double acc = 0.0;
+    for (int k = 0; k < list.n; ++k) {
+      if (list.at[k] != at) {
+        if (at >= 0) out[static_cast<long long>(at) * nb * nb + e] = acc;
+        at = list.at[k];
+        acc = out[static_cast<long long>(at) * nb * nb + e];
+      }
+      acc = __dadd_rn(acc, prod[k]);
+    }
+    out[static_cast<long long>(at) * nb * nb + e] = acc;
   }
 }
 
@@ -765,8 +810,9 @@ size_t smem_gamma() {
 
 template <int NBP>
 int node_impl(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s,
-              bool bf16) {
+              bool bf16, int nlm) {
   StageScope prof(c, ST_GRAM_NODE, 1, s);
+  const dim3 grid(gram_ctas(c, GK_NODE), nlm);
   if constexpr (NBP <= 20) {
     const unsigned char* f = reinterpret_cast<const unsigned char*>(alm);
     // the ring's bulk copies start on 16-byte boundaries
@@ -774,53 +820,60 @@ int node_impl(const zeta_ctx* c, const float* delta, const float* alm, double* p
     if (bf16) {  // bfloat16 fields, register-blocked float32 Gram (faster here than the tensor cores)
       const size_t smr = smem_node_rb<NBP, 1>();
       if (prep(k_gram_node_rb<NBP, 1>, smr)) return ZETA_ECUDA;
-      k_gram_node_rb<NBP, 1><<<gram_ctas(c, GK_NODE), kRbThreads, smr, s>>>(delta, f, c->ng, c->p.nbins, partials,
+      k_gram_node_rb<NBP, 1><<<grid, kRbThreads, smr, s>>>(delta, f, c->ng, c->p.nbins, partials,
                                                                            c->d_status);
     } else {
       const size_t smr = smem_node_rb<NBP, 0>();
       if (prep(k_gram_node_rb<NBP, 0>, smr)) return ZETA_ECUDA;
-      k_gram_node_rb<NBP, 0><<<gram_ctas(c, GK_NODE), kRbThreads, smr, s>>>(delta, f, c->ng, c->p.nbins, partials,
+      k_gram_node_rb<NBP, 0><<<grid, kRbThreads, smr, s>>>(delta, f, c->ng, c->p.nbins, partials,
                                                                            c->d_status);
     }
     return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
   }
-  if (bf16)  // bfloat16 fields with more than 20 bins: the tensor-core Gram (gram_ws.cu)
-    return launch_gram_ws(c, delta, alm, partials, gram_ctas(c, GK_NODE), 1, false, s);
+  if (bf16) {  // bfloat16 fields with more than 20 bins: the tensor-core Gram (gram_ws.cu), pair by pair
+    const size_t per = static_cast<size_t>(c->ng) * NBP / 2;  // floats of one pair's fields
+    for (int i = 0; i < nlm; ++i) {
+      const int rc = launch_gram_ws(c, delta, alm + i * per, partials + static_cast<size_t>(i) * grid.x * c->p.nbins * c->p.nbins,
+                                    grid.x, 1, false, s);
+      if (rc != ZETA_OK) return rc;
+    }
+    return ZETA_OK;
+  }
   const size_t sm = smem_node<NBP>();
   if (prep(k_gram_node<NBP>, sm)) return ZETA_ECUDA;
-  k_gram_node<NBP><<<gram_ctas(c, GK_NODE), kThreads, sm, s>>>(delta, reinterpret_cast<const float4*>(alm), c->ng,
+  k_gram_node<NBP><<<grid, kThreads, sm, s>>>(delta, reinterpret_cast<const float4*>(alm), c->ng,
                                                                  c->p.nbins, partials, c->d_status);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
 template <int NBP, int D>
-int gamma_impl(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s) {
+int gamma_impl(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s, int nlm) {
   StageScope prof(c, ST_GRAM_GAMMA, 1, s);
   const size_t sm = smem_gamma<NBP, D>();
   if (prep(k_gram_gamma<NBP, D>, sm)) return ZETA_ECUDA;
   if (c->gamma_q != GammaShape<NBP, D>::K) return ZETA_EINVAL;
-  k_gram_gamma<NBP, D><<<gram_ctas(c, GK_GAMMA), kThreads, sm, s>>>(
+  k_gram_gamma<NBP, D><<<dim3(gamma_ctas(c), nlm), kThreads, sm, s>>>(
       delta, reinterpret_cast<const float4*>(alm), c->ng, c->n, c->p.nbins, c->d_gq, partials);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
 template <int NBP>
-int mass_impl(const zeta_ctx* c, const unsigned long long* hist, int l, double* partials, cudaStream_t s) {
+int mass_impl(const zeta_ctx* c, const unsigned long long* hist, int l, double* partials, cudaStream_t s, int nl) {
   StageScope prof(c, ST_MASS, 1, s);
   const size_t sm = smem_mass<NBP>();
   if (prep(k_gram_mass<NBP>, sm)) return ZETA_ECUDA;
   const float* jt = c->d_jtab + static_cast<long long>(l) * c->nn2 * (4 * ((c->p.nbins + 3) / 4));
-  k_gram_mass<NBP><<<gram_ctas(c, GK_MASS), kThreads, sm, s>>>(hist, hist + c->nn2, jt, c->nn2, c->p.nbins, partials);
+  k_gram_mass<NBP><<<dim3(mass_ctas(c), nl), kThreads, sm, s>>>(hist, hist + c->nn2, jt, c->nn2, c->p.nbins, partials);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
 template <int NBP>
 int rows_rb_impl(const zeta_ctx* c, const float* pvals, const float4* s_tq, int64_t np, double* partials, int grid,
-                 cudaStream_t s) {
+                 cudaStream_t s, int nlm) {
   if constexpr (NBP <= 20) {
     const size_t smr = smem_node_rb<NBP, 2>();
     if (prep(k_gram_node_rb<NBP, 2>, smr)) return ZETA_ECUDA;
-    k_gram_node_rb<NBP, 2><<<grid, kRbThreads, smr, s>>>(reinterpret_cast<const float*>(s_tq),
+    k_gram_node_rb<NBP, 2><<<dim3(grid, nlm), kRbThreads, smr, s>>>(reinterpret_cast<const float*>(s_tq),
                                                          reinterpret_cast<const unsigned char*>(pvals), np,
                                                          c->p.nbins, partials, c->d_status);
     return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
@@ -831,8 +884,8 @@ int rows_rb_impl(const zeta_ctx* c, const float* pvals, const float4* s_tq, int6
 }  // namespace
 
 int launch_gram_rows_rb(const zeta_ctx* c, const float* pvals, const float4* s_tq, int64_t np, double* partials,
-                        int grid, cudaStream_t s) {
-#define ZK_CALL(P) rows_rb_impl<P>(c, pvals, s_tq, np, partials, grid, s)
+                        int grid, cudaStream_t s, int nlm) {
+#define ZK_CALL(P) rows_rb_impl<P>(c, pvals, s_tq, np, partials, grid, s, nlm)
   ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
 }
@@ -845,24 +898,36 @@ int gram_ctas(const zeta_ctx* c, int kind) {
   return g > kMaxCtas ? kMaxCtas : g;
 }
 
+// A tile per CTA at most, and a chunk of |n|^2 per CTA at most: more CTAs would only write zeros.
+int gamma_ctas(const zeta_ctx* c) {
+  const int g = gram_ctas(c, GK_GAMMA);
+  return g < c->ntiles ? g : static_cast<int>(c->ntiles);
+}
+int mass_ctas(const zeta_ctx* c) {
+  const long long chunks = (c->nn2 + kPB - 1) / kPB;
+  const int g = gram_ctas(c, GK_MASS);
+  return g < chunks ? g : static_cast<int>(chunks);
+}
+
 int launch_gram_node(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s,
-                     bool bf16) {
-#define ZK_CALL(P) node_impl<P>(c, delta, alm, partials, s, bf16)
+                     bool bf16, int nlm) {
+#define ZK_CALL(P) node_impl<P>(c, delta, alm, partials, s, bf16, nlm)
   ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
 }
 
-int launch_gram_gamma(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s) {
+int launch_gram_gamma(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s,
+                      int nlm) {
   if (c->p.dsup == 2) {
-#define ZK_CALL(P) gamma_impl<P, 2>(c, delta, alm, partials, s)
+#define ZK_CALL(P) gamma_impl<P, 2>(c, delta, alm, partials, s, nlm)
     ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
   } else if (c->p.dsup == 3) {
-#define ZK_CALL(P) gamma_impl<P, 5>(c, delta, alm, partials, s)
+#define ZK_CALL(P) gamma_impl<P, 5>(c, delta, alm, partials, s, nlm)
     ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
   } else {
-#define ZK_CALL(P) gamma_impl<P, 4>(c, delta, alm, partials, s)
+#define ZK_CALL(P) gamma_impl<P, 4>(c, delta, alm, partials, s, nlm)
     ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
   }
@@ -907,8 +972,8 @@ int launch_xi_hist(const zeta_ctx* c, const unsigned long long* hist, int nout, 
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
-int launch_mass(const zeta_ctx* c, const unsigned long long* hist, int l, double* partials, cudaStream_t s) {
-#define ZK_CALL(P) mass_impl<P>(c, hist, l, partials, s)
+int launch_mass(const zeta_ctx* c, const unsigned long long* hist, int l, double* partials, cudaStream_t s, int nl) {
+#define ZK_CALL(P) mass_impl<P>(c, hist, l, partials, s, nl)
   ZK_NBP_SWITCH(c->p.nbins, ZK_CALL)
 #undef ZK_CALL
 }
@@ -918,6 +983,14 @@ int launch_reduce(const zeta_ctx* c, const double* partials, int nparts, double 
   StageScope prof(c, ST_REDUCE, 1, s);
   const int nb = c->p.nbins;
   k_reduce<<<(nb * nb + 7) / 8, 256, 0, s>>>(partials, nparts, nb, scale, wdiv, out, store ? 1 : 0);
+  return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
+}
+
+int launch_reduce_list(const zeta_ctx* c, const double* partials, int nparts, const ReduceList& list, const double* wdiv,
+                       double* out, cudaStream_t s, bool store) {
+  StageScope prof(c, ST_REDUCE, 1, s);
+  const int nb = c->p.nbins;
+  k_reduce_list<<<nb * nb, 32 * list.n, 0, s>>>(partials, nparts, nb, list, wdiv, out, store ? 1 : 0);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 

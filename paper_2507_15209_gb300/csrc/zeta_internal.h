@@ -171,6 +171,17 @@ void profile_release(const zeta_ctx* c);
 // first time a kernel needs more (so later launches can be captured into a CUDA graph).
 int ensure_smem(const void* kernel, size_t bytes);
 
+// Pairs (l, m) that one launch takes together (small grids: see lm_batch).
+constexpr int kMaxLm = 16;
+struct LmList {
+  int n = 0;
+  signed char l[kMaxLm] = {}, m[kMaxLm] = {};
+  void add(int l_, int m_) {
+    l[n] = static_cast<signed char>(l_);
+    m[n++] = static_cast<signed char>(m_);
+  }
+};
+
 // ---- launchers (fft.cu) ----
 int set_ylm_constants();
 int launch_r2c(const zeta_ctx* c, const float* delta, float2* dhat, cudaStream_t s);
@@ -179,6 +190,9 @@ int launch_r2c(const zeta_ctx* c, const float* delta, float2* dhat, cudaStream_t
 // bf16: the groups are written as four bfloat16 per point ([g][z][y][x][4], 8 bytes) instead of float4
 int launch_alm(const zeta_ctx* c, const float2* dhat, int l, int m, int b0, int nf, float2* spec, float* out,
                cudaStream_t s, bool bf16 = false);
+// The fields of every pair of the list, one pair after the other in spec and out.
+int launch_alm_list(const zeta_ctx* c, const float2* dhat, const LmList& lms, int b0, int nf, float2* spec, float* out,
+                    cudaStream_t s, bool bf16 = false);
 // Adjoint of the reconstruction for nf bin-interleaved real fields h_b (bins 0..nf-1):
 // gk += sum_b (-1)^l K_lm,b DFT(h_b); spec is scratch for nf half spectra.
 int launch_adj_spectral(const zeta_ctx* c, const float* fields, int nf, float2* spec, int l, int m, float2* gk,
@@ -244,12 +258,15 @@ int launch_adj_finish_particles(const zeta_ctx* c, const float4* parts, int64_t 
 // ---- launchers (sums.cu) ----
 enum GramKind { GK_NODE = 0, GK_PART = 1, GK_GAMMA = 2, GK_MASS = 3, GK_TC = 4 };
 int gram_ctas(const zeta_ctx* c, int kind);
+// The Grams of nlm (l, m) pairs whose fields follow each other in alm; the partials of pair i start at
+// i * (the form's CTAs per pair) * nbins^2.  gamma_ctas: CTAs per pair of the Gamma form.
 int launch_gram_node(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s,
-                     bool bf16 = false);
+                     bool bf16 = false, int nlm = 1);
+int gamma_ctas(const zeta_ctx* c);
 int launch_gram_gamma(const zeta_ctx* c, const float* delta, const float* alm, double* partials,
-                      cudaStream_t s);
+                      cudaStream_t s, int nlm = 1);
 int launch_gram_particles(const zeta_ctx* c, const int* s_cell, const float4* s_tq, const int64_t* tile_start,
-                          int64_t np, const float* alm, float* pvals, double* partials, cudaStream_t s);
+                          int64_t np, const float* alm, float* pvals, double* partials, cudaStream_t s, int nlm = 1);
 // Bytes of the interpolated particle rows [np][bins padded to 4] that launch_gram_particles uses.
 size_t particle_rows_bytes(const zeta_ctx* c, int64_t np);
 // tensor-core node Gram (gram_tc.cu), arithmetic chosen by c->p.gram
@@ -274,16 +291,27 @@ int launch_reduce_vec(const zeta_ctx* c, const double* partials, int nparts, con
 // Particle form of the 2PCF: interpolated rows of the l = 0 fields, then per-CTA sums of w f_b.
 int launch_particle_xi(const zeta_ctx* c, const int* s_cell, const float4* s_tq, const int64_t* tile_start,
                        int64_t np, const float* alm, float* pvals, double* partials, cudaStream_t s);
-int launch_mass(const zeta_ctx* c, const unsigned long long* hist, int l, double* partials, cudaStream_t s);
+// nl multipoles from l on, mass_ctas partials each
+int mass_ctas(const zeta_ctx* c);
+int launch_mass(const zeta_ctx* c, const unsigned long long* hist, int l, double* partials, cudaStream_t s, int nl = 1);
 // Weighted Gram of the interpolated particle rows ([np][bins padded to 4]) with the weights of the
 // prepared records, register-blocked (<= 20 bins; ZETA_ENOTSUP above): grid CTAs, partials[grid].
 int launch_gram_rows_rb(const zeta_ctx* c, const float* pvals, const float4* s_tq, int64_t np, double* partials,
-                        int grid, cudaStream_t s);
+                        int grid, cudaStream_t s, int nlm = 1);
 // Number of per-CTA partial Grams launch_gram_particles writes.
 int gram_particle_parts(const zeta_ctx* c);
 // out[b1][b2] += scale * (1/ *wdiv if wdiv) * sum_cta partials[cta][b1][b2], symmetrised.
 int launch_reduce(const zeta_ctx* c, const double* partials, int nparts, double scale, const double* wdiv,
                   double* out, cudaStream_t s, bool store = false);
+// The same for several contributions at once (nparts partials each, one after the other in partials), added in
+// the order of the list: out[at[i] nb^2 + ..] += (or, with store, =) scale[i] (/ *wdiv) * sum.
+struct ReduceList {
+  int n = 0;
+  int at[kMaxLm] = {};
+  double scale[kMaxLm] = {};
+};
+int launch_reduce_list(const zeta_ctx* c, const double* partials, int nparts, const ReduceList& list, const double* wdiv,
+                       double* out, cudaStream_t s, bool store);
 // zeta[f][l] = per-(l, m) slots summed in the full measurement's order (see zeta_reduce_lm).
 int launch_reduce_lm(const zeta_ctx* c, const double* slots, int nforms, int part_form, double* zeta, cudaStream_t s);
 
