@@ -584,7 +584,7 @@ int zeta_xi(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
   if (forms & ZETA_SUM_NODE) {
     unsigned long long* hist = at<unsigned long long>(c, L.mhist);
     ZK_TRY(launch_mass_hist(c, dhat, hist, stream, c->d_phi));
-    ZK_TRY(launch_xi_hist(c, hist, nb, nullptr, xi + f * nb, stream));
+    ZK_TRY(launch_xi_hist(c, hist, nb, nullptr, part, xi + f * nb, stream));
     ++f;
   }
   if (want_p) {
@@ -628,7 +628,7 @@ int zeta_xi_radii(zeta_ctx* c, const float* delta_hat, int nr, const double* rad
     return ZETA_ECUDA;
   unsigned long long* hist = at<unsigned long long>(c, L.mhist);
   ZK_TRY(launch_mass_hist(c, reinterpret_cast<const float2*>(delta_hat), hist, stream, c->d_phi));
-  ZK_TRY(launch_xi_hist(c, hist, nr, dr, xi, stream));
+  ZK_TRY(launch_xi_hist(c, hist, nr, dr, at<double>(c, L.partials), xi, stream));
   // the host array must stay valid until the copy has been read
   return cudaStreamSynchronize(stream) == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }

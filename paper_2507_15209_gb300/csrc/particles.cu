@@ -630,7 +630,7 @@ int part_impl(const zeta_ctx* c, const int* s_cell, const float4* s_tq, const in
 template <int NBP>
 __global__ void __launch_bounds__(kThreads) k_row_sums(const float* __restrict__ pvals, const float4* __restrict__ s_tq,
                                                        long long np, int nb, double* __restrict__ partials) {
-  __shared__ double red[kThreads];
+  __shared__ double red[kThreads / 32][NBP];
   double dacc[NBP];
   float acc[NBP];
 #pragma unroll
@@ -660,17 +660,19 @@ __global__ void __launch_bounds__(kThreads) k_row_sums(const float* __restrict__
       pending = 0;
     }
   }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int b = 0; b < NBP; ++b) {
-    if (b >= nb) break;  // uniform across the CTA
-    red[threadIdx.x] = dacc[b] + static_cast<double>(acc[b]);
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-      if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) partials[static_cast<long long>(blockIdx.x) * nb + b] = red[0];
-    __syncthreads();
+  for (int b = 0; b < NBP; ++b) {  // fixed butterfly over the lanes, then the warps in order
+    double v = dacc[b] + static_cast<double>(acc[b]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (lane == 0) red[warp][b] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < nb) {
+    double v = red[0][threadIdx.x];
+    for (int w = 1; w < kThreads / 32; ++w) v += red[w][threadIdx.x];
+    partials[static_cast<long long>(blockIdx.x) * nb + threadIdx.x] = v;
   }
 }
 

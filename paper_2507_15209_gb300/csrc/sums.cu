@@ -13,6 +13,7 @@
 // shared by all of them is in gram.cuh.
 #include <utility>
 
+#include "cell.cuh"
 #include "gram.cuh"
 
 namespace zk {
@@ -566,66 +567,343 @@ __global__ void __launch_bounds__(kThreads)
   cta_store<NBP>(g, red, nb, partials + static_cast<long long>(blockIdx.x) * nb * nb);
 }
 
+// Gamma form of the cubic B-spline and Daubechies bases for up to 20 bins: the batches, their order and all
+// arithmetic of k_gram_gamma, with the x pass taken out of the batch.  A tile is walked layer by layer and
+// row by row; the x-filtered values of the D stencil rows of the current row of cells (8 K points each, D
+// planes) are kept in a ring, and going to the next row filters one new stencil row per plane instead of
+// D^2 rows per batch, from coalesced loads (lanes along x).  The y pass of a batch reads the ring, and since
+// its buffer, the value table and the ring are three, a batch takes two barriers instead of four.  Bound:
+// shared-memory wavefronts and issue.  128^3, 15 bins, cubic: 8689 us with k_gram_gamma, ROWS_FIGURES.
+template <int NBP, int D>
+struct GammaRows {
+  using S = GammaShape<NBP, D>;
+  static constexpr int OZS = D * kTile * 5 + 5;  // float4 per plane of the ring (5 mod 8: distinct banks)
+  static constexpr int RING = S::NCH * D * OZS * 4;  // floats
+  static constexpr size_t BYTES = static_cast<size_t>(RING + S::YF + S::VF) * sizeof(float);
+};
+
+template <int NBP, int D>
+__global__ void __launch_bounds__(kThreads)
+    k_gram_gamma_rows(const float* __restrict__ delta, const float4* __restrict__ f4, long long ng, int n, int nb,
+                      const float* __restrict__ gq, double* __restrict__ partials) {
+  using G = Gram<NBP>;
+  using S = GammaShape<NBP, D>;
+  using R = GammaRows<NBP, D>;
+  constexpr int K = S::K, NC = S::NC, OFF = S::OFF, OZS = R::OZS;
+  static_assert(NC == 2 && K == 5, "batches of two cells along x");
+  extern __shared__ __align__(16) unsigned char smraw[];
+  f4 += static_cast<long long>(blockIdx.y) * ((nb + 3) / 4) * ng;  // blockIdx.y: (l, m) pair
+  partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
+  float* vals = reinterpret_cast<float*>(smraw);                       // [kPB][NBS]
+  float* wts = vals + kPB * G::NBS;                                     // [kPB]
+  float4* ybuf = reinterpret_cast<float4*>(vals + S::VF);              // [ch][cell][oz][ky][kx]
+  float4* ring = reinterpret_cast<float4*>(vals + S::VF + S::YF);      // [ch][oz] (OZS) [row mod D][8 K]
+  double* red = reinterpret_cast<double*>(smraw);                      // reused after the main loop
+  const int pr = threadIdx.x % G::NPAIR, grp = threadIdx.x / G::NPAIR;
+  int b1 = 0, b2 = 0;
+  pair_blocks(pr, G::NBLK, b1, b2);
+  GramAcc<NBP> g;
+  g.init();
+  float fm[D][K], qw[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    qw[k] = __ldg(gq + k);
+#pragma unroll
+    for (int o = 0; o < D; ++o) fm[o][k] = __ldg(gq + K + k * D + o);
+  }
+  const int ngrp = (nb + 3) / 4;
+  const int nch = ngrp + (S::DB ? 0 : 1);
+  const int nt = n / kTile;
+  const long long ntiles = static_cast<long long>(nt) * nt * nt;
+  const int mask = n - 1;
+  for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int tx = static_cast<int>(t % nt), ty = static_cast<int>((t / nt) % nt),
+              tz = static_cast<int>(t / (static_cast<long long>(nt) * nt));
+    for (int lyr = 0; lyr < kTile * kTile; ++lyr) {
+      const int y = lyr % kTile, cz = tz * kTile + lyr / kTile, cy = ty * kTile + y;
+      // x pass: the new stencil rows of the D planes (at y = 0 all D, else the last); the y passes that read
+      // the slots before are behind a barrier
+      const int r0 = y == 0 ? 0 : D - 1;
+      for (int i = threadIdx.x; i < nch * D * (D - r0) * kTile; i += kThreads) {
+        const int c = i % kTile, oz = (i / kTile) % D, q = i / (kTile * D);
+        const int ch = q % nch, oy = r0 + q / nch;
+        const int x0 = tx * kTile + c - OFF;
+        const long long row = (static_cast<long long>((cz - OFF + oz) & mask) * n + ((cy - OFF + oy) & mask)) * n;
+        float4 in[D];
+        if (ch < ngrp) {
+          const float4* base = f4 + ch * ng + row;
+#pragma unroll
+          for (int e = 0; e < D; ++e) in[e] = __ldg(base + ((x0 + e) & mask));
+        } else {
+#pragma unroll
+          for (int e = 0; e < D; ++e) in[e] = make_float4(__ldg(delta + row + ((x0 + e) & mask)), 0.f, 0.f, 0.f);
+        }
+        float4* out = ring + (ch * D + oz) * OZS + ((y + oy) % D) * (kTile * K) + c * K;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int o = 0; o < D; ++o) {
+            v.x = fmaf(fm[o][k], in[o].x, v.x);
+            v.y = fmaf(fm[o][k], in[o].y, v.y);
+            v.z = fmaf(fm[o][k], in[o].z, v.z);
+            v.w = fmaf(fm[o][k], in[o].w, v.w);
+          }
+          out[k] = v;
+        }
+      }
+      __syncthreads();
+      for (int xb = 0; xb < kTile / NC; ++xb) {
+        // y pass: task (channel, cell, oz, kx) filters D x-filtered values into K
+        for (int i = threadIdx.x; i < nch * NC * D * K; i += kThreads) {
+          const int kx = i % K, r = i / K;
+          const int oz = r % D, j = (r / D) % NC, ch = r / (D * NC);
+          const float4* src = ring + (ch * D + oz) * OZS + (xb * NC + j) * K + kx;
+          float4 in[D];
+#pragma unroll
+          for (int o = 0; o < D; ++o) in[o] = src[((y + o) % D) * (kTile * K)];
+          float4* out = ybuf + r * S::YR + kx;
+#pragma unroll
+          for (int k = 0; k < K; ++k) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int o = 0; o < D; ++o) {
+              v.x = fmaf(fm[o][k], in[o].x, v.x);
+              v.y = fmaf(fm[o][k], in[o].y, v.y);
+              v.z = fmaf(fm[o][k], in[o].z, v.z);
+              v.w = fmaf(fm[o][k], in[o].w, v.w);
+            }
+            out[k * K] = v;
+          }
+        }
+        __syncthreads();  // the previous batch's contraction is done with the value table as well
+        // z pass: task (channel, cell, ky, kx) filters D y-pass values into the K points along z
+        for (int i = threadIdx.x; i < nch * NC * K * K; i += kThreads) {
+          const int kk = i % (K * K), r = i / (K * K);
+          const int j = r % NC, ch = r / NC;
+          const int kx = kk % K, ky = kk / K;
+          const float4* src = ybuf + r * D * S::YR + kk;
+          float4 in[D];
+#pragma unroll
+          for (int o = 0; o < D; ++o) in[o] = src[o * S::YR];
+          const float wxy = __ldg(gq + kx) * __ldg(gq + ky);
+          float dn = 0.f;
+          if (S::DB && ch == 0)  // delta at the node itself
+            dn = __ldg(delta + (static_cast<long long>(cz) * n + cy) * n + tx * kTile + xb * NC + j);
+#pragma unroll
+          for (int k = 0; k < K; ++k) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int o = 0; o < D; ++o) {
+              v.x = fmaf(fm[o][k], in[o].x, v.x);
+              v.y = fmaf(fm[o][k], in[o].y, v.y);
+              v.z = fmaf(fm[o][k], in[o].z, v.z);
+              v.w = fmaf(fm[o][k], in[o].w, v.w);
+            }
+            const int p = j * S::K3 + k * K * K + kk;
+            const float w = wxy * qw[k];
+            if (ch < ngrp) *reinterpret_cast<float4*>(vals + p * G::NBS + 4 * ch) = v;
+            else wts[p] = w * v.x;  // n_rec at the point
+            if (S::DB && ch == 0) wts[p] = w * dn;
+          }
+        }
+        __syncthreads();
+        if (grp < G::NGRP) g.add(vals, wts, NC * S::K3, b1, b2, grp);
+      }
+    }
+  }
+  __syncthreads();
+  cta_store<NBP>(g, red, nb, partials + static_cast<long long>(blockIdx.x) * nb * nb);
+}
+
+// Gamma form of the linear B-spline: the batches (32 cells, 8 points each), their order and all arithmetic of
+// k_gram_gamma, but one thread takes a cell's eight nodes of one channel through the three passes in
+// registers (lanes along x, so the loads are coalesced), and two batches share a round: two barriers per
+// two batches instead of four per batch, and no pass buffers.  64^3, 8 bins: 72 us per (l, m) with
+// k_gram_gamma (eight pairs per launch), LIN_FIGURES.
+template <int NBP>
+struct GammaLin {
+  static constexpr int BATCHES = 2;
+  static constexpr int POINTS = BATCHES * kPB;
+  static constexpr size_t BYTES = static_cast<size_t>(POINTS) * (Gram<NBP>::NBS + 1) * sizeof(float);
+};
+
+template <int NBP>
+__global__ void __launch_bounds__(kThreads)
+    k_gram_gamma_lin(const float* __restrict__ delta, const float4* __restrict__ f4, long long ng, int n, int nb,
+                     const float* __restrict__ gq, double* __restrict__ partials) {
+  using G = Gram<NBP>;
+  using L = GammaLin<NBP>;
+  constexpr int NC = kPB / 8, ROUND = NC * L::BATCHES;  // cells per batch and per round
+  extern __shared__ __align__(16) unsigned char smraw[];
+  f4 += static_cast<long long>(blockIdx.y) * ((nb + 3) / 4) * ng;  // blockIdx.y: (l, m) pair
+  partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
+  float* vals = reinterpret_cast<float*>(smraw);  // [POINTS][NBS]
+  float* wts = vals + L::POINTS * G::NBS;          // [POINTS]
+  double* red = reinterpret_cast<double*>(smraw);  // reused after the main loop
+  const int pr = threadIdx.x % G::NPAIR, grp = threadIdx.x / G::NPAIR;
+  int b1 = 0, b2 = 0;
+  pair_blocks(pr, G::NBLK, b1, b2);
+  GramAcc<NBP> g;
+  g.init();
+  float fm[2][2], qw[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    qw[k] = __ldg(gq + k);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) fm[o][k] = __ldg(gq + 2 + k * 2 + o);
+  }
+  const int ngrp = (nb + 3) / 4;
+  const int nt = n / kTile;
+  const long long ntiles = static_cast<long long>(nt) * nt * nt;
+  const int mask = n - 1;
+  auto filt = [&](int k, float4 a, float4 b) {
+    return make_float4(fmaf(fm[1][k], b.x, fmaf(fm[0][k], a.x, 0.f)), fmaf(fm[1][k], b.y, fmaf(fm[0][k], a.y, 0.f)),
+                       fmaf(fm[1][k], b.z, fmaf(fm[0][k], a.z, 0.f)), fmaf(fm[1][k], b.w, fmaf(fm[0][k], a.w, 0.f)));
+  };
+  for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int tx = static_cast<int>(t % nt), ty = static_cast<int>((t / nt) % nt),
+              tz = static_cast<int>(t / (static_cast<long long>(nt) * nt));
+    for (int rd = 0; rd < kTile * kTile * kTile / ROUND; ++rd) {
+      __syncthreads();  // the previous round's contraction is done with the value table
+      for (int i = threadIdx.x; i < (ngrp + 1) * ROUND; i += kThreads) {
+        const int j = i % ROUND, ch = i / ROUND, ci = rd * ROUND + j;
+        const int cx = tx * kTile + ci % kTile, cy = ty * kTile + (ci / kTile) % kTile, cz = tz * kTile + ci / (kTile * kTile);
+        const int xs[2] = {cx, (cx + 1) & mask};
+        float4 v[2][2][2];  // [z][y][x]: nodes, then filtered along x, y, z
+#pragma unroll
+        for (int oz = 0; oz < 2; ++oz)
+#pragma unroll
+          for (int oy = 0; oy < 2; ++oy) {
+            const long long row = (static_cast<long long>((cz + oz) & mask) * n + ((cy + oy) & mask)) * n;
+#pragma unroll
+            for (int ox = 0; ox < 2; ++ox)
+              v[oz][oy][ox] = ch < ngrp ? __ldg(f4 + ch * ng + row + xs[ox])
+                                        : make_float4(__ldg(delta + row + xs[ox]), 0.f, 0.f, 0.f);
+          }
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+#pragma unroll
+          for (int y = 0; y < 2; ++y) {
+            const float4 a = v[z][y][0], b = v[z][y][1];
+            v[z][y][0] = filt(0, a, b);
+            v[z][y][1] = filt(1, a, b);
+          }
+#pragma unroll
+        for (int z = 0; z < 2; ++z)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const float4 a = v[z][0][x], b = v[z][1][x];
+            v[z][0][x] = filt(0, a, b);
+            v[z][1][x] = filt(1, a, b);
+          }
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const float wxy = qw[x] * qw[y];
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+              const float4 r = filt(z, v[0][y][x], v[1][y][x]);
+              const int p = j * 8 + z * 4 + y * 2 + x;
+              if (ch < ngrp) *reinterpret_cast<float4*>(vals + p * G::NBS + 4 * ch) = r;
+              else wts[p] = (wxy * qw[z]) * r.x;  // n_rec at the point
+            }
+          }
+      }
+      __syncthreads();
+      if (grp < G::NGRP)
+#pragma unroll 1
+        for (int b = 0; b < L::BATCHES; ++b) g.add(vals + b * kPB * G::NBS, wts + b * kPB, kPB, b1, b2, grp);
+    }
+  }
+  __syncthreads();
+  cta_store<NBP>(g, red, nb, partials + static_cast<long long>(blockIdx.x) * nb * nb);
+}
+
 // ---------------------------------------------------------------------------------------
 // Uniform term of the particle form: U_l[b1][b2] = (2l+1)/(4 pi) sum_k w(k) J_l,b1(|n|^2)
 // J_l,b2(|n|^2), w = (1, or 2 off the ix = 0 plane) |delta_hat|^2 Mhat over the stored half
 // spectrum without its Nyquist planes.  The window depends on the mode only through the
 // integer |n|^2, so w is summed per |n|^2 once per catalogue and each l is then a Gram over
 // the 3 (n/2 - 1)^2 + 1 values of |n|^2 (Nyquist planes excluded).  The per-|n|^2 sums are
-// 64-bit fixed point in units of max(w) 2^-48: integer atomics, so the sums do not depend on
-// the order of the modes, and a value of |n|^2 holds far fewer than 2^16 modes, so no sum can
-// overflow.
-constexpr double kMassUnit = 281474976710656.0;  // 2^48
+// 64-bit fixed point in units of 2^-52 of a bound on w: integer atomics, so the sums do not
+// depend on the order of the modes; a mode is below 2^52 units and a value of |n|^2 holds at most
+// 2980 of them (512^3), so no sum reaches 2^64.
+//
+// The unit comes from F, the power of two above the largest |Re|, |Im| of delta_hat (Mhat <= 1, so w <= 4 F^2):
+// one streaming pass of integer maxima over float bits.  The weights themselves are float32 pairs (products
+// by FMA, sums by two-sum: about 46 bits) turned into integers by integer instructions, and the up to
+// four modes (+-n_y, +-n_z) of one |n|^2 are added before one atomic.  256^3: 175 + 214 us with float64
+// weights (the float64 pipe retires two operations per SM and clock) and one atomic per mode,
+// 27 + 44 us now.
+constexpr int kMassBits = 52;
 
-__device__ __forceinline__ bool mass_mode(long long i, int n, const float2* __restrict__ dhat,
-                                          const float* __restrict__ mhat, double& w, long long& n2) {
-  const int nc = n / 2;
-  const int ix = static_cast<int>(i % nc), iy = static_cast<int>((i / nc) % n),
-            iz = static_cast<int>(i / (static_cast<long long>(nc) * n));
-  if (iy == n / 2 || iz == n / 2) return false;
-  const int fy = iy < n / 2 ? iy : iy - n, fz = iz < n / 2 ? iz : iz - n;
-  n2 = static_cast<long long>(ix) * ix + fy * fy + fz * fz;
-  const float2 d = dhat[i];
-  w = (ix == 0 ? 1.0 : 2.0) * (static_cast<double>(d.x) * d.x + static_cast<double>(d.y) * d.y) *
-      (static_cast<double>(mhat[ix]) * mhat[iy] * mhat[iz]);
-  return true;
+// 4 F^2 of the bits that k_mass_max left (0, infinity and NaN pass through)
+__device__ __forceinline__ double mass_bound(const unsigned long long* amax_bits) {
+  const unsigned b = static_cast<unsigned>(*amax_bits);
+  const double f = __uint_as_float(b);
+  if (b == 0 || b >= 0x7f800000u) return 4.0 * f * f;
+  int e;
+  frexp(f, &e);  // f < 2^e
+  return ldexp(4.0, 2 * e);
+}
+__device__ __forceinline__ double mass_unit(const unsigned long long* amax_bits) {
+  return ldexp(mass_bound(amax_bits), -kMassBits);
 }
 
-// max_k w(k) as the bits of a non-negative double (their unsigned order is the numeric order)
-__global__ void k_mass_max(const float2* __restrict__ dhat, const float* __restrict__ mhat, int n,
-                           unsigned long long* __restrict__ wmax_bits) {
-  const long long total = static_cast<long long>(n) * n * (n / 2);
-  unsigned long long m = 0;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
-       i += static_cast<long long>(blockDim.x) * gridDim.x) {
-    double w;
-    long long n2;
-    if (mass_mode(i, n, dhat, mhat, w, n2)) {
-      const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(w));
-      m = b > m ? b : m;
-    }
+// max over the half spectrum of the bits of |Re| and |Im| (their unsigned order is the numeric order, NaN last)
+__global__ void __launch_bounds__(kThreads) k_mass_max(const uint2* __restrict__ dhat, long long total,
+                                                       unsigned long long* __restrict__ amax_bits) {
+  unsigned m = 0;
+  // total is a multiple of 4 kThreads only from 32^3 on; the caller's array is 8-byte aligned
+  const long long step = static_cast<long long>(blockDim.x) * gridDim.x;
+  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total; i += 4 * step) {
+    uint2 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = i + u * step < total ? dhat[i + u * step] : make_uint2(0u, 0u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) m = max(m, max(v[u].x & 0x7fffffffu, v[u].y & 0x7fffffffu));
   }
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, off);
-    m = o > m ? o : m;
-  }
-  if ((threadIdx.x & 31) == 0) atomicMax(wmax_bits, m);
+  for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned*>(amax_bits), m);  // the low word (little endian)
 }
 
-__global__ void k_mass_hist(const float2* __restrict__ dhat, const float* __restrict__ mhat, int n,
-                            const unsigned long long* __restrict__ wmax_bits, unsigned long long* __restrict__ hist) {
-  const double wmax = __longlong_as_double(static_cast<long long>(*wmax_bits));
-  if (!(wmax > 0.0)) return;
-  const double scale = kMassUnit / wmax;
-  const long long total = static_cast<long long>(n) * n * (n / 2);
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
-       i += static_cast<long long>(blockDim.x) * gridDim.x) {
-    double w;
-    long long n2;
-    if (mass_mode(i, n, dhat, mhat, w, n2)) {
-      const unsigned long long q = __double2ull_rn(w * scale);
-      if (q) atomicAdd(hist + n2, q);
+// One warp per (|n_y|, |n_z|), lanes along n_x.
+__global__ void __launch_bounds__(kThreads) k_mass_hist(const float2* __restrict__ dhat, const float* __restrict__ mhat,
+                                                        int n, const unsigned long long* __restrict__ amax_bits,
+                                                        unsigned long long* __restrict__ hist) {
+  const unsigned ab = static_cast<unsigned>(*amax_bits);
+  if (ab == 0 || ab >= 0x7f800000u) return;  // nothing, or not finite: the unit says so
+  int e;
+  frexp(static_cast<double>(__uint_as_float(ab)), &e);
+  const int nc = n / 2;
+  const int lane = threadIdx.x & 31;
+  // powers of two in two steps, so that neither is out of range: x 2^-e is at most 1
+  const float s1 = ldexpf(1.f, -e / 2), s2 = ldexpf(1.f, -(e - e / 2));
+  for (int row = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < nc * nc; row += gridDim.x * (kThreads / 32)) {
+    const int fy = row % nc, fz = row / nc;
+    const float mz = mhat[fz], my = mhat[fy];  // Mhat is even
+    const float yzh = my * mz, yzl = fmaf(my, mz, -yzh);
+    for (int ix = lane; ix < nc; ix += 32) {
+      const float mx = mhat[ix];
+      const float mh = mx * yzh, ml = fmaf(mx, yzh, -mh) + mx * yzl;
+      unsigned long long sum = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (((k & 1) && fy == 0) || ((k & 2) && fz == 0)) continue;
+        const int iy = (k & 1) ? n - fy : fy, iz = (k & 2) ? n - fz : fz;
+        const float2 d = dhat[(static_cast<long long>(iz) * n + iy) * nc + ix];
+        const float x = d.x * s1 * s2, y = d.y * s1 * s2;
+        const float p = x * x, q = y * y, pe = fmaf(x, x, -p), qe = fmaf(y, y, -q);
+        const float h = p + q, bb = h - p;
+        const float l = ((p - (h - bb)) + (q - bb)) + (pe + qe);  // x^2 + y^2 = h + l <= 2
+        const float w = h * mh, wl = fmaf(h, mh, -w) + fmaf(h, ml, l * mh);
+        sum += static_cast<unsigned long long>(fix64_prod(w, 1.f, kMassBits - 2) + fix64_prod(wl, 1.f, kMassBits - 2));
+      }
+      if (ix > 0) sum *= 2;  // the mirrored half
+      if (sum) atomicAdd(hist + (ix * ix + fy * fy + fz * fz), sum);
     }
   }
 }
@@ -633,7 +911,7 @@ __global__ void k_mass_hist(const float2* __restrict__ dhat, const float* __rest
 // Gram of one l over the values of |n|^2: weight S(|n|^2), values J_l,b(|n|^2)
 template <int NBP>
 __global__ void __launch_bounds__(kThreads) k_gram_mass(const unsigned long long* __restrict__ hist,
-                                                        const unsigned long long* __restrict__ wmax_bits,
+                                                        const unsigned long long* __restrict__ amax_bits,
                                                         const float* __restrict__ jt, long long nn2, int nb,
                                                         double* __restrict__ partials) {
   using G = Gram<NBP>;
@@ -648,7 +926,7 @@ __global__ void __launch_bounds__(kThreads) k_gram_mass(const unsigned long long
   pair_blocks(pr, G::NBLK, b1, b2);
   GramAcc<NBP> g;
   g.init();
-  const double unit = __longlong_as_double(static_cast<long long>(*wmax_bits)) / kMassUnit;
+  const double unit = mass_unit(amax_bits);
   const int nbp = 4 * ((nb + 3) / 4);
   const long long nchunk = (nn2 + kPB - 1) / kPB;
   for (long long ch = blockIdx.x; ch < nchunk; ch += gridDim.x) {
@@ -755,16 +1033,15 @@ __global__ void k_reduce_lm(const double* __restrict__ slots, int nforms, int pa
 // a fixed stride of |n|^2 in float64 and the CTA reduces in a fixed order.
 // mode 0: out[b] for the bins, radial factor from the window table (l = 0 row);
 // mode 1: out[i] for radii[i], radial factor j_0(k r_i) W_TH(k rsec).
-__global__ void __launch_bounds__(256) k_xi_hist(const unsigned long long* __restrict__ hist,
-                                                 const unsigned long long* __restrict__ wmax_bits, long long nn2,
+// Each output is split over gridDim.y CTAs (a stride of |n|^2 each) whose partial sums k_xi_final adds.
+__global__ void __launch_bounds__(256) k_xi_hist(const unsigned long long* __restrict__ hist, long long nn2,
                                                  const float* __restrict__ jt0, int nbp, const float* __restrict__ wprim,
                                                  double ng, double kunit, const double* __restrict__ radii,
-                                                 double rsec, int mode, double* __restrict__ out) {
-  __shared__ double red[256];
-  const double unit = __longlong_as_double(static_cast<long long>(*wmax_bits)) / kMassUnit;
+                                                 double rsec, int mode, double* __restrict__ part) {
+  __shared__ double red[8];
   const int o = blockIdx.x;
   double acc = 0.0;
-  for (long long i = threadIdx.x; i < nn2; i += blockDim.x) {
+  for (long long i = blockIdx.y * 256LL + threadIdx.x; i < nn2; i += 256LL * gridDim.y) {
     const unsigned long long h = hist[i];
     if (!h) continue;
     double f;
@@ -782,13 +1059,22 @@ __global__ void __launch_bounds__(256) k_xi_hist(const unsigned long long* __res
     if (wprim) f *= static_cast<double>(__ldg(wprim + i)) * ng;
     acc += static_cast<double>(h) * f;
   }
-  red[threadIdx.x] = acc;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) acc += red[i];
+    part[blockIdx.y * gridDim.x + o] = acc;
   }
-  if (threadIdx.x == 0) out[o] = red[0] * unit / (ng * ng);
+}
+__global__ void k_xi_final(const double* __restrict__ part, int nout, int nsplit,
+                           const unsigned long long* __restrict__ amax_bits, double ng, double* __restrict__ out) {
+  const int o = blockIdx.x * blockDim.x + threadIdx.x;
+  if (o >= nout) return;
+  double sum = 0.0;
+  for (int k = 0; k < nsplit; ++k) sum += part[k * nout + o];
+  out[o] = sum * mass_unit(amax_bits) / (ng * ng);
 }
 
 template <int NBP>
@@ -849,11 +1135,22 @@ int node_impl(const zeta_ctx* c, const float* delta, const float* alm, double* p
 template <int NBP, int D>
 int gamma_impl(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s, int nlm) {
   StageScope prof(c, ST_GRAM_GAMMA, 1, s);
-  const size_t sm = smem_gamma<NBP, D>();
-  if (prep(k_gram_gamma<NBP, D>, sm)) return ZETA_ECUDA;
   if (c->gamma_q != GammaShape<NBP, D>::K) return ZETA_EINVAL;
-  k_gram_gamma<NBP, D><<<dim3(gamma_ctas(c), nlm), kThreads, sm, s>>>(
-      delta, reinterpret_cast<const float4*>(alm), c->ng, c->n, c->p.nbins, c->d_gq, partials);
+  const float4* f4 = reinterpret_cast<const float4*>(alm);
+  const dim3 grid(gamma_ctas(c), nlm);
+  if constexpr (D == 2) {
+    const size_t main = GammaLin<NBP>::BYTES, sm = main > red_bytes<NBP>() ? main : red_bytes<NBP>();
+    if (prep(k_gram_gamma_lin<NBP>, sm)) return ZETA_ECUDA;
+    k_gram_gamma_lin<NBP><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
+  } else if constexpr (NBP <= 20) {
+    const size_t main = GammaRows<NBP, D>::BYTES, sm = main > red_bytes<NBP>() ? main : red_bytes<NBP>();
+    if (prep(k_gram_gamma_rows<NBP, D>, sm)) return ZETA_ECUDA;
+    k_gram_gamma_rows<NBP, D><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
+  } else {  // the row ring of more bins would leave one CTA per SM
+    const size_t sm = smem_gamma<NBP, D>();
+    if (prep(k_gram_gamma<NBP, D>, sm)) return ZETA_ECUDA;
+    k_gram_gamma<NBP, D><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
+  }
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
@@ -936,39 +1233,49 @@ int launch_gram_gamma(const zeta_ctx* c, const float* delta, const float* alm, d
 int launch_mass_hist(const zeta_ctx* c, const float2* dhat, unsigned long long* hist, cudaStream_t s,
                      const float* table1d) {
   StageScope prof(c, ST_MASS, 2, s);
-  // hist[0 .. nn2) the fixed-point sums, hist[nn2] the bits of max w
+  // hist[0 .. nn2) the fixed-point sums, hist[nn2] the bits of the largest component
   if (cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (c->nn2 + 1), s) != cudaSuccess) return ZETA_ECUDA;
-  const int grid = c->num_sms * 8;
   const float* t = table1d ? table1d : c->d_mhat;
-  k_mass_max<<<grid, kThreads, 0, s>>>(dhat, t, c->n, hist + c->nn2);
-  k_mass_hist<<<grid, kThreads, 0, s>>>(dhat, t, c->n, hist + c->nn2, hist);
+  k_mass_max<<<c->num_sms * 8, kThreads, 0, s>>>(reinterpret_cast<const uint2*>(dhat), c->ng / 2, hist + c->nn2);
+  const int rows = c->nc * c->nc;
+  const int grid = (rows + kThreads / 32 - 1) / (kThreads / 32);
+  k_mass_hist<<<grid < c->num_sms * 16 ? grid : c->num_sms * 16, kThreads, 0, s>>>(dhat, t, c->n, hist + c->nn2, hist);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
-// out[b] = (1 / *wdiv) sum_cta partials[cta][b], the CTAs in order (one thread per b).
+// out[b] = (1 / *wdiv) sum_cta partials[cta][b]: one warp per b, lane j the CTAs j, j + 32, .. in order, then a
+// fixed butterfly.
 __global__ void k_reduce_vec(const double* __restrict__ part, int nparts, int nb, const double* __restrict__ wdiv,
                              double* __restrict__ out) {
-  const int b = threadIdx.x;
-  if (b >= nb) return;
+  const int b = blockIdx.x;
   double sum = 0.0;
-  for (int k = 0; k < nparts; ++k) sum += part[static_cast<long long>(k) * nb + b];
-  out[b] = sum / *wdiv;
+  for (int k = threadIdx.x; k < nparts; k += 32) sum += part[static_cast<long long>(k) * nb + b];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+  if (threadIdx.x == 0) out[b] = sum / *wdiv;
 }
 
 int launch_reduce_vec(const zeta_ctx* c, const double* partials, int nparts, const double* wdiv, double* out,
                       cudaStream_t s) {
   StageScope prof(c, ST_REDUCE, 1, s);
-  k_reduce_vec<<<1, 32, 0, s>>>(partials, nparts, c->p.nbins, wdiv, out);
+  k_reduce_vec<<<c->p.nbins, 32, 0, s>>>(partials, nparts, c->p.nbins, wdiv, out);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
-int launch_xi_hist(const zeta_ctx* c, const unsigned long long* hist, int nout, const double* radii, double* out,
-                   cudaStream_t s) {
-  StageScope prof(c, ST_MASS, 1, s);
+int launch_xi_hist(const zeta_ctx* c, const unsigned long long* hist, int nout, const double* radii, double* part,
+                   double* out, cudaStream_t s) {
+  StageScope prof(c, ST_MASS, 2, s);
   const int nbp = 4 * ((c->p.nbins + 3) / 4);
   const double kunit = 2.0 * 3.14159265358979323846 / c->p.box;
-  k_xi_hist<<<nout, 256, 0, s>>>(hist, hist + c->nn2, c->nn2, c->d_jtab, nbp, c->d_wprim, static_cast<double>(c->ng),
-                                 kunit, radii, c->p.tophat, radii ? 1 : 0, out);
+  const double ng = static_cast<double>(c->ng);
+  // CTAs per output: four per SM in all, a chunk of 256 values of |n|^2 each at least (15 outputs at 256^3: 185 us
+  // with one CTA per output, 13 + 6 us)
+  int split = 4 * c->num_sms / nout;
+  const int most = static_cast<int>((c->nn2 + 255) / 256);
+  split = split < 1 ? 1 : split > most ? most : split;
+  k_xi_hist<<<dim3(nout, split), 256, 0, s>>>(hist, c->nn2, c->d_jtab, nbp, c->d_wprim, ng, kunit, radii, c->p.tophat,
+                                              radii ? 1 : 0, part);
+  k_xi_final<<<(nout + 127) / 128, 128, 0, s>>>(part, nout, split, hist + c->nn2, ng, out);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 

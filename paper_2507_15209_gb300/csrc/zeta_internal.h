@@ -283,8 +283,9 @@ int launch_mass_hist(const zeta_ctx* c, const float2* dhat, unsigned long long* 
                      const float* table1d = nullptr);
 // 2PCF from a histogram of (1 or 2) |delta_hat|^2 Phi-hat per |n|^2 (launch_mass_hist with c->d_phi):
 // radii == nullptr: out[b] for the bins (nout = nbins); else out[i] at the point radii (device).
-int launch_xi_hist(const zeta_ctx* c, const unsigned long long* hist, int nout, const double* radii, double* out,
-                   cudaStream_t s);
+// part: scratch of kMaxCtas doubles (nout <= kMaxCtas)
+int launch_xi_hist(const zeta_ctx* c, const unsigned long long* hist, int nout, const double* radii, double* part,
+                   double* out, cudaStream_t s);
 // out[b] = sum_cta partials[cta][b] / *wdiv (fixed order)
 int launch_reduce_vec(const zeta_ctx* c, const double* partials, int nparts, const double* wdiv, double* out,
                       cudaStream_t s);
