@@ -170,9 +170,10 @@ __global__ void __launch_bounds__(kAT) k_adj_mass(const float2* __restrict__ dha
 // lanes by shuffles; the direct term sum_b c_b grad f_b is added to the particle's slot; and c is
 // scattered with the assignment stencil by float4 atomics.  Bound: L2 atomics and gathers.  256^3, 1M
 // particles, 10 bins, D = 4: 2167 us with one thread per particle and bin group (values and gradients
-// through shared memory), 974 us now.
+// through shared memory), 974 with
+// the sixteen rows unrolled (spills at two CTAs per SM), about 835 with rolled layers and three.
 template <int NBP, int D>
-__global__ void __launch_bounds__(kAT, 2)
+__global__ void __launch_bounds__(kAT, 3)
     k_adj_points(const int* __restrict__ s_cell, const float4* __restrict__ s_tq, const int* __restrict__ sidx,
                  long long np, const float4* __restrict__ f4, long long ng, int n, int nb, float hinv,
                  const float* __restrict__ S, const double* __restrict__ wsum, float4* __restrict__ h4,
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(kAT, 2)
     bs_w<D>(t.y, wy, dy);
     bs_w<D>(t.z, wz, dz);
     const int cx = (cell & mask) - OFF, cy = ((cell >> lg) & mask) - OFF, cz = (cell >> (2 * lg)) - OFF;
-    constexpr int NR = D == 4 ? 16 : 2;  // rows: (oz, oy) for D = 4, oz for D = 2
+    constexpr int NY = D == 4 ? 4 : 1;  // stencil rows of a z-layer that a lane takes
     const int ox = D == 4 ? li : (li & 1);
     float lx = wx[0], ldx = dx[0];  // this lane's x factor (for D = 2 times the y factor)
 #pragma unroll
@@ -210,27 +211,43 @@ __global__ void __launch_bounds__(kAT, 2)
     const int xo = (cx + ox) & mask;
     const bool y1 = li >> 1;
     const float ly = y1 ? wy[1] : wy[0], ldy = y1 ? dy[1] : dy[0];  // D = 2 only
-    auto row_at = [&](int r) {
-      const int oz = D == 4 ? r >> 2 : r, oy = D == 4 ? r & 3 : static_cast<int>(y1);
-      return (((((cz + oz) & mask) << lg) + ((cy + oy) & mask)) << lg) + xo;
+    int yo[NY];
+#pragma unroll
+    for (int o = 0; o < NY; ++o) yo[o] = (((cy + (D == 4 ? o : static_cast<int>(y1))) & mask) << lg) + xo;
+    // the layers are a rolled loop: unrolled, the row addresses and weight products of all sixteen rows
+    // stay in registers over the bin groups and spill
+    auto layer = [&](int oz, float& w, float& d) {
+      w = wz[0];
+      d = dz[0];
+#pragma unroll
+      for (int o = 1; o < D; ++o) {
+        w = oz == o ? wz[o] : w;
+        d = oz == o ? dz[o] : d;
+      }
+      return ((cz + oz) & mask) << (2 * lg);
     };
     float f[G], gx[G], gy[G], gz[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       const float4* src = f4 + g * ng;
       float vp[4] = {0.f, 0.f, 0.f, 0.f}, vy[4] = {0.f, 0.f, 0.f, 0.f}, vz[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+      for (int oz = 0; oz < D; ++oz) {
+        float wo, zo;
+        const int at = layer(oz, wo, zo);
+        float4 vr[NY];
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const float4 v = __ldg(src + row_at(r));
-        const float vv[4] = {v.x, v.y, v.z, v.w};
-        const int oz = D == 4 ? r >> 2 : r, oy = D == 4 ? r & 3 : 0;
-        const float a = D == 4 ? wz[oz] * wy[oy] : wz[oz], az = D == 4 ? dz[oz] * wy[oy] : dz[oz];
-        const float ay = D == 4 ? wz[oz] * dy[oy] : 0.f;
+        for (int oy = 0; oy < NY; ++oy) vr[oy] = __ldg(src + (at + yo[oy]));
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          vp[j] = fmaf(a, vv[j], vp[j]);
-          vz[j] = fmaf(az, vv[j], vz[j]);
-          if (D == 4) vy[j] = fmaf(ay, vv[j], vy[j]);
+        for (int oy = 0; oy < NY; ++oy) {
+          const float vv[4] = {vr[oy].x, vr[oy].y, vr[oy].z, vr[oy].w};
+          const float a = D == 4 ? wo * wy[oy] : wo, az = D == 4 ? zo * wy[oy] : zo, ay = D == 4 ? wo * dy[oy] : 0.f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            vp[j] = fmaf(a, vv[j], vp[j]);
+            vz[j] = fmaf(az, vv[j], vz[j]);
+            if (D == 4) vy[j] = fmaf(ay, vv[j], vy[j]);
+          }
         }
       }
       float k4[4][4];  // [kind][bin]: f, df/dx, df/dy, df/dz of this lane's nodes
@@ -306,11 +323,15 @@ __global__ void __launch_bounds__(kAT, 2)
       for (int j = 0; j < 4; ++j) cb[j] = __shfl_sync(0xffffffffu, c[g], l0 + j);
       if (act && t.w != 0.f) {
         float4* dst = h4 + g * ng;
+#pragma unroll 1
+        for (int oz = 0; oz < D; ++oz) {
+          float wo, zo;
+          const int at = layer(oz, wo, zo);
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          const int oz = D == 4 ? r >> 2 : r, oy = D == 4 ? r & 3 : 0;
-          const float a = (D == 4 ? wz[oz] * wy[oy] : wz[oz] * ly) * lx;
-          atomicAdd(dst + row_at(r), make_float4(a * cb[0], a * cb[1], a * cb[2], a * cb[3]));
+          for (int oy = 0; oy < NY; ++oy) {
+            const float a = (D == 4 ? wo * wy[oy] : wo * ly) * lx;
+            atomicAdd(dst + (at + yo[oy]), make_float4(a * cb[0], a * cb[1], a * cb[2], a * cb[3]));
+          }
         }
       }
     }
