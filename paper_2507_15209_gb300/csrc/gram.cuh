@@ -107,8 +107,8 @@ struct GramAcc {
   // vals: [npts][NBS] shared, wts: [npts] shared.  This thread takes points grp, grp + NGRP,
   // ...; the float32 partials are flushed before a call that would take them past kFlush
   // points (a call brings at most kPB / NGRP <= kFlush points), so the loop itself is
-  // flush-free and U points are in flight at a time.
-  template <int U = 2>
+  // flush-free and U points are in flight at a time.  PAD: floats between groups of eight points' rows.
+  template <int U = 2, int PAD = 0>
   __device__ __forceinline__ void add(const float* vals, const float* wts, int npts, int b1, int b2, int grp) {
     constexpr int NG = Gram<NBP, NT>::NGRP;
     constexpr int NBS = Gram<NBP, NT>::NBS;
@@ -116,21 +116,22 @@ struct GramAcc {
     if (pending + count > kFlush) flush();
     pending += count;
     int pt = grp;
+    auto row = [&](int p) { return vals + p * NBS + (PAD ? (p >> 3) * PAD : 0); };
     for (; pt + (U - 1) * NG < npts; pt += U * NG) {
       float w[U];
       float4 x[U], y[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         w[u] = wts[pt + u * NG];
-        x[u] = *reinterpret_cast<const float4*>(vals + (pt + u * NG) * NBS + 4 * b1);
-        y[u] = *reinterpret_cast<const float4*>(vals + (pt + u * NG) * NBS + 4 * b2);
+        x[u] = *reinterpret_cast<const float4*>(row(pt + u * NG) + 4 * b1);
+        y[u] = *reinterpret_cast<const float4*>(row(pt + u * NG) + 4 * b2);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) accum(x[u], y[u], w[u]);
     }
     for (; pt < npts; pt += NG) {
-      const float4 x = *reinterpret_cast<const float4*>(vals + pt * NBS + 4 * b1);
-      const float4 y = *reinterpret_cast<const float4*>(vals + pt * NBS + 4 * b2);
+      const float4 x = *reinterpret_cast<const float4*>(row(pt) + 4 * b1);
+      const float4 y = *reinterpret_cast<const float4*>(row(pt) + 4 * b2);
       accum(x, y, wts[pt]);
     }
   }

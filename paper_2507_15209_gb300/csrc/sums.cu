@@ -720,13 +720,18 @@ __global__ void __launch_bounds__(kThreads)
 // Gamma form of the linear B-spline: the batches (32 cells, 8 points each), their order and all arithmetic of
 // k_gram_gamma, but one thread takes a cell's eight nodes of one channel through the three passes in
 // registers (lanes along x, so the loads are coalesced), and two batches share a round: two barriers per
-// two batches instead of four per batch, and no pass buffers.  64^3, 8 bins: 72 us per (l, m) with
-// k_gram_gamma (eight pairs per launch), 54 here.
+// two batches instead of four per batch, and no pass buffers.  us per (l, m), k_gram_gamma -> here: 3 bins at
+// 32^3 53 -> 39; 8 at 64^3 89 -> 61, at 256^3 3810 -> 1983.
+// Up to 12 bins the channels of a round (bins in fours, and delta) fit its threads; with more, a mostly idle
+// second pass over them makes it slower on large grids (256^3: 15 bins 5810 -> 6660, 20 bins 7210 -> 7545).
 template <int NBP>
 struct GammaLin {
   static constexpr int BATCHES = 2;
   static constexpr int POINTS = BATCHES * kPB;
-  static constexpr size_t BYTES = static_cast<size_t>(POINTS) * (Gram<NBP>::NBS + 1) * sizeof(float);
+  // a float4 between the rows of two cells, so that the lanes' rows, a cell apart, hit distinct banks
+  static constexpr int PAD = 4;
+  static constexpr int VALS = POINTS * Gram<NBP>::NBS + POINTS / 8 * PAD;
+  static constexpr size_t BYTES = static_cast<size_t>(VALS + POINTS) * sizeof(float);
 };
 
 template <int NBP>
@@ -740,7 +745,7 @@ __global__ void __launch_bounds__(kThreads)
   f4 += static_cast<long long>(blockIdx.y) * ((nb + 3) / 4) * ng;  // blockIdx.y: (l, m) pair
   partials += static_cast<long long>(blockIdx.y) * gridDim.x * nb * nb;
   float* vals = reinterpret_cast<float*>(smraw);  // [POINTS][NBS]
-  float* wts = vals + L::POINTS * G::NBS;          // [POINTS]
+  float* wts = vals + L::VALS;                     // [POINTS]
   double* red = reinterpret_cast<double*>(smraw);  // reused after the main loop
   const int pr = threadIdx.x % G::NPAIR, grp = threadIdx.x / G::NPAIR;
   int b1 = 0, b2 = 0;
@@ -807,7 +812,7 @@ __global__ void __launch_bounds__(kThreads)
             for (int z = 0; z < 2; ++z) {
               const float4 r = filt(z, v[0][y][x], v[1][y][x]);
               const int p = j * 8 + z * 4 + y * 2 + x;
-              if (ch < ngrp) *reinterpret_cast<float4*>(vals + p * G::NBS + 4 * ch) = r;
+              if (ch < ngrp) *reinterpret_cast<float4*>(vals + p * G::NBS + j * L::PAD + 4 * ch) = r;
               else wts[p] = (wxy * qw[z]) * r.x;  // n_rec at the point
             }
           }
@@ -815,7 +820,8 @@ __global__ void __launch_bounds__(kThreads)
       __syncthreads();
       if (grp < G::NGRP)
 #pragma unroll 1
-        for (int b = 0; b < L::BATCHES; ++b) g.add(vals + b * kPB * G::NBS, wts + b * kPB, kPB, b1, b2, grp);
+        for (int b = 0; b < L::BATCHES; ++b)
+          g.template add<2, L::PAD>(vals + b * (L::VALS / L::BATCHES), wts + b * kPB, kPB, b1, b2, grp);
     }
   }
   __syncthreads();
@@ -1139,15 +1145,15 @@ int gamma_impl(const zeta_ctx* c, const float* delta, const float* alm, double* 
   if (c->gamma_q != GammaShape<NBP, D>::K) return ZETA_EINVAL;
   const float4* f4 = reinterpret_cast<const float4*>(alm);
   const dim3 grid(gamma_ctas(c), nlm);
-  if constexpr (D == 2) {
+  if constexpr (D == 2 && NBP <= 12) {  // 128^3, 12 bins: 634 us with k_gram_gamma, 554; more bins: see GammaLin
     const size_t main = GammaLin<NBP>::BYTES, sm = main > red_bytes<NBP>() ? main : red_bytes<NBP>();
     if (prep(k_gram_gamma_lin<NBP>, sm)) return ZETA_ECUDA;
     k_gram_gamma_lin<NBP><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
-  } else if constexpr (NBP <= 20) {
+  } else if constexpr (D > 2 && NBP <= 20) {
     const size_t main = GammaRows<NBP, D>::BYTES, sm = main > red_bytes<NBP>() ? main : red_bytes<NBP>();
     if (prep(k_gram_gamma_rows<NBP, D>, sm)) return ZETA_ECUDA;
     k_gram_gamma_rows<NBP, D><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
-  } else {  // the row ring of more bins would leave one CTA per SM
+  } else {  // more bins; with D > 2 their row ring would leave one CTA per SM
     const size_t sm = smem_gamma<NBP, D>();
     if (prep(k_gram_gamma<NBP, D>, sm)) return ZETA_ECUDA;
     k_gram_gamma<NBP, D><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
