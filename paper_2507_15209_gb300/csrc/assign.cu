@@ -270,38 +270,6 @@ __global__ void __launch_bounds__(256) k_assign_scatter(const float4* __restrict
   }
 }
 
-// v inv - 1 for a 64-bit integer v, rounded to float32, equal to the float64 formula's value: with
-// inv = ih + il and v as the float32 values of its leading and following 24 bits, the product and the
-// difference are float32 pairs within 2^-45 (|v inv| + 1); a result that close to a rounding boundary
-// (one in 10^5, or any much smaller than 1) takes the float64 formula.  That formula for every node
-// (three conversions, two operations) took 118 us for 256^3 nodes, bound by the float64 pipe; this 41 us.
-__device__ __forceinline__ float contrast_of(long long v, float ih, float il, double inv) {
-  const bool neg = v < 0;
-  const unsigned long long a = neg ? 0ULL - static_cast<unsigned long long>(v) : static_cast<unsigned long long>(v);
-  if (a == 0) return -1.f;
-  const int lz = __clzll(static_cast<long long>(a));
-  const unsigned long long m = a << lz;
-  const float sc = __uint_as_float(static_cast<uint32_t>(127 + 40 - lz) << 23);  // 2^(40 - lz)
-  float hi = static_cast<float>(static_cast<uint32_t>(m >> 40)) * sc;
-  float lo = static_cast<float>(static_cast<uint32_t>(m >> 16) & 0xffffffu) * (sc * 5.9604644775390625e-8f);
-  if (neg) {
-    hi = -hi;
-    lo = -lo;
-  }
-  const float p = hi * ih;
-  const float e = fmaf(hi, ih, -p) + fmaf(hi, il, lo * ih);
-  const float s = p - 1.f, bb = s - p;
-  const float rest = ((p - (s - bb)) + (-1.f - bb)) + e;
-  const float r = s + rest;
-  const float miss = fabsf((s - r) + rest);  // r is off by this much
-  const float size = fabsf(p) + 1.f, tol = size * 5.684341886080802e-14f;  // 2^-44 (|p| + 1)
-  const uint32_t rb = __float_as_uint(r);
-  const float h = __uint_as_float((rb & 0x7f800000u) - (24u << 23));  // half a unit in the last place
-  const bool near = fabsf(miss - h) < tol || ((rb & 0x7fffffu) == 0 && fabsf(miss - 0.5f * h) < tol);
-  if (near || fabsf(r) < size * 2.44140625e-4f) return static_cast<float>(static_cast<double>(v) * inv - 1.0);
-  return r;
-}
-
 __global__ void k_assign_finalize(const unsigned long long* __restrict__ acc, long long ng,
                                   const double* __restrict__ wstat, float* __restrict__ delta) {
   const float2 f = *reinterpret_cast<const float2*>(wstat + 3);
@@ -316,8 +284,8 @@ __global__ void k_assign_finalize(const unsigned long long* __restrict__ acc, lo
       d0 = contrast_of(v0, f.x, f.y, inv);
       d1 = contrast_of(v1, f.x, f.y, inv);
     } else {
-      d0 = static_cast<float>(static_cast<double>(v0) * inv - 1.0);
-      d1 = static_cast<float>(static_cast<double>(v1) * inv - 1.0);
+      d0 = contrast_f64(v0, inv);
+      d1 = contrast_f64(v1, inv);
     }
     delta[i] = d0;
     delta[i + 1] = d1;
