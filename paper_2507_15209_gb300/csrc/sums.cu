@@ -13,8 +13,8 @@
 // shared by all of them is in gram.cuh.
 #include <utility>
 
-#include "cell.cuh"
 #include "gram.cuh"
+#include "mass.cuh"
 
 namespace zk {
 namespace {
@@ -834,91 +834,97 @@ __global__ void __launch_bounds__(kThreads)
 // spectrum without its Nyquist planes.  The window depends on the mode only through the
 // integer |n|^2, so w is summed per |n|^2 once per catalogue and each l is then a Gram over
 // the 3 (n/2 - 1)^2 + 1 values of |n|^2 (Nyquist planes excluded).  The per-|n|^2 sums are
-// 64-bit fixed point in units of 2^-52 of a bound on w: integer atomics, so the sums do not
-// depend on the order of the modes; a mode is below 2^52 units and a value of |n|^2 holds at most
-// 2980 of them (512^3), so no sum reaches 2^64.
+// 64-bit fixed point in units of 2^-52 of the power of two above the largest w: integer atomics, so the
+// sums do not depend on the order of the modes; a mode is at most 2^52 units and a value of |n|^2 holds
+// at most 2980 of them (512^3), so no sum reaches 2^64.
 //
-// The unit comes from F, the power of two above the largest |Re|, |Im| of delta_hat (Mhat <= 1, so w <= 4 F^2):
-// one streaming pass of integer maxima over float bits.  The weights themselves are float32 pairs (products
-// by FMA, sums by two-sum: about 46 bits) turned into integers by integer instructions, and the up to
-// four modes (+-n_y, +-n_z) of one |n|^2 are added before one atomic.  256^3: 175 + 214 us with float64
-// weights (the float64 pipe retires two operations per SM and clock) and one atomic per mode,
-// 27 + 44 us now.
+// One pass finds that power of two (from float32 weights where those are in range: their error only makes it
+// the next one) and a second forms the sums from integer weights (mass.cuh), with one table product for the
+// up to four modes (+-n_y, +-n_z) of one |n|^2, which are added before one atomic.  A whole mass_term,
+// us: 256^3 422 with float64 weights (that pipe retires two operations per SM and clock) and one atomic per
+// mode, 84 now; 512^3 3059, 398.
 constexpr int kMassBits = 52;
+// The word behind the sums: 0 without a positive weight, kMassBad with a non-finite mode, else 2048 plus the
+// exponent of the power of two.
+constexpr unsigned kMassBias = 2048, kMassBad = 0xffffu;
 
-// 4 F^2 of the bits that k_mass_max left (0, infinity and NaN pass through)
-__device__ __forceinline__ double mass_bound(const unsigned long long* amax_bits) {
-  const unsigned b = static_cast<unsigned>(*amax_bits);
-  const double f = __uint_as_float(b);
-  if (b == 0 || b >= 0x7f800000u) return 4.0 * f * f;
-  int e;
-  frexp(f, &e);  // f < 2^e
-  return ldexp(4.0, 2 * e);
-}
-__device__ __forceinline__ double mass_unit(const unsigned long long* amax_bits) {
-  return ldexp(mass_bound(amax_bits), -kMassBits);
+__device__ __forceinline__ double mass_unit(const unsigned long long* top) {
+  const unsigned t = static_cast<unsigned>(*top);
+  if (t == 0) return 0.0;
+  if (t == kMassBad) return __longlong_as_double(0x7ff8000000000000LL);
+  return ldexp(1.0, static_cast<int>(t) - static_cast<int>(kMassBias) - kMassBits);
 }
 
-// max over the half spectrum of the bits of |Re| and |Im| (their unsigned order is the numeric order, NaN last)
-__global__ void __launch_bounds__(kThreads) k_mass_max(const uint2* __restrict__ dhat, long long total,
-                                                       unsigned long long* __restrict__ amax_bits) {
-  unsigned m = 0;
-  // total is a multiple of 4 kThreads only from 32^3 on; the caller's array is 8-byte aligned
-  const long long step = static_cast<long long>(blockDim.x) * gridDim.x;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total; i += 4 * step) {
-    uint2 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = i + u * step < total ? dhat[i + u * step] : make_uint2(0u, 0u);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) m = max(m, max(v[u].x & 0x7fffffffu, v[u].y & 0x7fffffffu));
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned*>(amax_bits), m);  // the low word (little endian)
-}
-
-// One warp per (|n_y|, |n_z|), lanes along n_x.
-__global__ void __launch_bounds__(kThreads) k_mass_hist(const float2* __restrict__ dhat, const float* __restrict__ mhat,
-                                                        int n, const unsigned long long* __restrict__ amax_bits,
-                                                        unsigned long long* __restrict__ hist) {
-  const unsigned ab = static_cast<unsigned>(*amax_bits);
-  if (ab == 0 || ab >= 0x7f800000u) return;  // nothing, or not finite: the unit says so
-  int e;
-  frexp(static_cast<double>(__uint_as_float(ab)), &e);
-  const int nc = n / 2;
-  const int lane = threadIdx.x & 31;
-  // powers of two in two steps, so that neither is out of range: x 2^-e is at most 1
-  const float s1 = ldexpf(1.f, -e / 2), s2 = ldexpf(1.f, -(e - e / 2));
+// Calls f(n_x, |n|^2, the three table values, the modes, 0 where there is none) for every group of up to four
+// modes (+-n_y, +-n_z); one warp per (|n_y|, |n_z|), lanes along n_x.
+template <typename F>
+__device__ __forceinline__ void mass_modes(const float2* __restrict__ dhat, const float* __restrict__ mhat, int n, F f) {
+  const int nc = n / 2, lane = threadIdx.x & 31;
   for (int row = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < nc * nc; row += gridDim.x * (kThreads / 32)) {
     const int fy = row % nc, fz = row / nc;
-    const float mz = mhat[fz], my = mhat[fy];  // Mhat is even
-    const float yzh = my * mz, yzl = fmaf(my, mz, -yzh);
+    const float mz = mhat[fz], my = mhat[fy];  // the tables are even
     for (int ix = lane; ix < nc; ix += 32) {
-      const float mx = mhat[ix];
-      const float mh = mx * yzh, ml = fmaf(mx, yzh, -mh) + mx * yzl;
-      unsigned long long sum = 0;
+      float2 d[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (((k & 1) && fy == 0) || ((k & 2) && fz == 0)) continue;
+        const bool on = !((k & 1) && fy == 0) && !((k & 2) && fz == 0);
         const int iy = (k & 1) ? n - fy : fy, iz = (k & 2) ? n - fz : fz;
-        const float2 d = dhat[(static_cast<long long>(iz) * n + iy) * nc + ix];
-        const float x = d.x * s1 * s2, y = d.y * s1 * s2;
-        const float p = x * x, q = y * y, pe = fmaf(x, x, -p), qe = fmaf(y, y, -q);
-        const float h = p + q, bb = h - p;
-        const float l = ((p - (h - bb)) + (q - bb)) + (pe + qe);  // x^2 + y^2 = h + l <= 2
-        const float w = h * mh, wl = fmaf(h, mh, -w) + fmaf(h, ml, l * mh);
-        sum += static_cast<unsigned long long>(fix64_prod(w, 1.f, kMassBits - 2) + fix64_prod(wl, 1.f, kMassBits - 2));
+        d[k] = on ? dhat[(static_cast<long long>(iz) * n + iy) * nc + ix] : make_float2(0.f, 0.f);
       }
-      if (ix > 0) sum *= 2;  // the mirrored half
-      if (sum) atomicAdd(hist + (ix * ix + fy * fy + fz * fz), sum);
+      f(ix, ix * ix + fy * fy + fz * fz, mhat[ix], my, mz, d);
     }
   }
+}
+
+__global__ void __launch_bounds__(kThreads) k_mass_max(const float2* __restrict__ dhat, const float* __restrict__ mhat,
+                                                       int n, unsigned long long* __restrict__ top) {
+  unsigned t = 0;
+  float fast = 0.f;
+  mass_modes(dhat, mhat, n, [&](int ix, int, float mx, float my, float mz, const float2(&d)[4]) {
+    const float m = mx * my * mz * (ix > 0 ? 2.f : 1.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t big = max(__float_as_uint(d[k].x) & 0x7fffffffu, __float_as_uint(d[k].y) & 0x7fffffffu);
+      // from 2^-40 to 2^62 the float32 weight neither over- nor underflows (the tables are above 2^-45)
+      if (big - 0x2b800000u < 0x33000000u) {
+        fast = fmaxf(fast, fmaf(d[k].x, d[k].x, d[k].y * d[k].y) * m);
+      } else if (big >= 0x7f800000u) {
+        t = kMassBad;
+      } else if (big) {
+        const WideFactor w = mode_weight(d[k].x, d[k].y, wide_product(my, mz, mx), ix > 0);
+        if (w.m) t = max(t, static_cast<unsigned>(wide_ceil(w) + static_cast<int>(kMassBias)));
+      }
+    }
+  });
+  if (fast > 0.f) {  // within 2^-20 of the exact weight: the power of two above both
+    int e;
+    frexp(static_cast<double>(fast) * 1.000001, &e);
+    t = max(t, static_cast<unsigned>(e + static_cast<int>(kMassBias)));
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) t = max(t, __shfl_xor_sync(0xffffffffu, t, off));
+  if ((threadIdx.x & 31) == 0 && t) atomicMax(reinterpret_cast<unsigned*>(top), t);  // the low word (little endian)
+}
+
+__global__ void __launch_bounds__(kThreads) k_mass_hist(const float2* __restrict__ dhat, const float* __restrict__ mhat,
+                                                        int n, const unsigned long long* __restrict__ top,
+                                                        unsigned long long* __restrict__ hist) {
+  const unsigned t = static_cast<unsigned>(*top);
+  if (t == 0 || t == kMassBad) return;  // nothing, or not finite: the unit says so
+  const int unit = static_cast<int>(t) - static_cast<int>(kMassBias) - kMassBits;
+  mass_modes(dhat, mhat, n, [&](int ix, int n2, float mx, float my, float mz, const float2(&d)[4]) {
+    const WideFactor m = wide_product(my, mz, mx);
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sum += wide_units(mode_weight(d[k].x, d[k].y, m, ix > 0), unit);
+    if (sum) atomicAdd(hist + n2, sum);
+  });
 }
 
 // Gram of one l over the values of |n|^2: weight S(|n|^2), values J_l,b(|n|^2)
 template <int NBP>
 __global__ void __launch_bounds__(kThreads) k_gram_mass(const unsigned long long* __restrict__ hist,
-                                                        const unsigned long long* __restrict__ amax_bits,
+                                                        const unsigned long long* __restrict__ top,
                                                         const float* __restrict__ jt, long long nn2, int nb,
                                                         double* __restrict__ partials) {
   using G = Gram<NBP>;
@@ -933,7 +939,7 @@ __global__ void __launch_bounds__(kThreads) k_gram_mass(const unsigned long long
   pair_blocks(pr, G::NBLK, b1, b2);
   GramAcc<NBP> g;
   g.init();
-  const double unit = mass_unit(amax_bits);
+  const double unit = mass_unit(top);
   const int nbp = 4 * ((nb + 3) / 4);
   const long long nchunk = (nn2 + kPB - 1) / kPB;
   for (long long ch = blockIdx.x; ch < nchunk; ch += gridDim.x) {
@@ -1076,12 +1082,12 @@ __global__ void __launch_bounds__(256) k_xi_hist(const unsigned long long* __res
   }
 }
 __global__ void k_xi_final(const double* __restrict__ part, int nout, int nsplit,
-                           const unsigned long long* __restrict__ amax_bits, double ng, double* __restrict__ out) {
+                           const unsigned long long* __restrict__ top, double ng, double* __restrict__ out) {
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= nout) return;
   double sum = 0.0;
   for (int k = 0; k < nsplit; ++k) sum += part[k * nout + o];
-  out[o] = sum * mass_unit(amax_bits) / (ng * ng);
+  out[o] = sum * mass_unit(top) / (ng * ng);
 }
 
 template <int NBP>
@@ -1240,13 +1246,14 @@ int launch_gram_gamma(const zeta_ctx* c, const float* delta, const float* alm, d
 int launch_mass_hist(const zeta_ctx* c, const float2* dhat, unsigned long long* hist, cudaStream_t s,
                      const float* table1d) {
   StageScope prof(c, ST_MASS, 2, s);
-  // hist[0 .. nn2) the fixed-point sums, hist[nn2] the bits of the largest component
+  // hist[0 .. nn2) the fixed-point sums, hist[nn2] the exponent of their unit
   if (cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (c->nn2 + 1), s) != cudaSuccess) return ZETA_ECUDA;
   const float* t = table1d ? table1d : c->d_mhat;
-  k_mass_max<<<c->num_sms * 8, kThreads, 0, s>>>(reinterpret_cast<const uint2*>(dhat), c->ng / 2, hist + c->nn2);
   const int rows = c->nc * c->nc;
-  const int grid = (rows + kThreads / 32 - 1) / (kThreads / 32);
-  k_mass_hist<<<grid < c->num_sms * 16 ? grid : c->num_sms * 16, kThreads, 0, s>>>(dhat, t, c->n, hist + c->nn2, hist);
+  int grid = (rows + kThreads / 32 - 1) / (kThreads / 32);
+  if (grid > c->num_sms * 16) grid = c->num_sms * 16;
+  k_mass_max<<<grid, kThreads, 0, s>>>(dhat, t, c->n, hist + c->nn2);
+  k_mass_hist<<<grid, kThreads, 0, s>>>(dhat, t, c->n, hist + c->nn2, hist);
   return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
 }
 
