@@ -72,7 +72,7 @@ enum {
   ZETA_ENOMEM = -3,     /* device allocation of the context's tables failed         */
   ZETA_ETIMEOUT = -4,   /* a bounded device wait gave up                            */
   ZETA_ENOTSUP = -5,    /* configuration not supported by this build                */
-  ZETA_EWORKSPACE = -6, /* workspace missing or smaller than zeta_workspace_bytes   */
+  ZETA_EWORKSPACE = -6, /* workspace missing or too small (see zeta_workspace_bytes) */
   ZETA_EDATA = -7       /* device found invalid input data (non-finite particle)    */
 };
 
@@ -157,11 +157,14 @@ int zeta_create(const zeta_params* p, zeta_ctx** out);
 /* Free the context and its device tables.  NULL is accepted. */
 int zeta_destroy(zeta_ctx* ctx);
 
-/* Bytes of workspace that zeta_zeta_ell needs for up to np_max particles and the given
- * summation forms; it also covers every single-step call.  0 on invalid arguments. */
+/* Bytes of workspace for zeta_zeta_ell with up to np_max particles and the given summation forms; it
+ * also covers every single-step call.  On grids up to 128^3 it has room for up to 16 (l, m) pairs at a
+ * time (128 MB of spectra and fields, 64 MB of interpolated rows), which then share launches; a
+ * smaller workspace is accepted as long as one pair fits (the size with lmax = 0), with fewer pairs
+ * per launch and the same results.  0 on invalid arguments. */
 size_t zeta_workspace_bytes(const zeta_ctx* ctx, int64_t np_max, int forms);
 
-/* Hand the context a caller-owned device workspace (256-byte aligned, >= the size above).
+/* Hand the context a caller-owned device workspace (256-byte aligned, of the size above; see there).
  * The library keeps the pointer, never frees it. */
 int zeta_set_workspace(zeta_ctx* ctx, void* dptr, size_t bytes);
 
@@ -309,7 +312,8 @@ int zeta_backward_particles(zeta_ctx* ctx, const float* particles, int64_t np, c
  * catalogue; when it holds k >= 2 whole per-catalogue workspaces (k times
  * zeta_workspace_bytes(ctx, largest np, forms), k <= 4), k catalogues run concurrently: the
  * graph forks k streams, and catalogue i runs on stream i mod k in slice i mod k of the
- * workspace (the catalogues share no data, so their kernels overlap where the GPU has room).
+ * workspace (the catalogues share no data, so their kernels overlap where the GPU has room).  In
+ * a workspace smaller than one of these, k is the number that fit with one (l, m) pair at a time.
  * Results do not depend on k.  Changing the workspace or the tuning drops the cached graph. */
 int zeta_batch(zeta_ctx* ctx, const float* particles, const int64_t* offsets, int ncat, int forms, double* zeta,
                zeta_stream stream);

@@ -21,13 +21,14 @@ struct Layout {
   // backward (gradient) regions
   size_t gk = 0, q = 0, wts = 0, hfield = 0, direct = 0, sidx = 0;
   size_t total = 0;
+  int pairs = 1;  // (l, m) pairs that the spectra and fields have room for
 };
 
 // (l, m) pairs that a measurement takes together.  On small grids every kernel of one pair is a few
 // microseconds of latency on a machine that is mostly idle, so the pairs share launches as long as their
 // spectra and fields stay within 128 MB, an L2's worth (64^3 with 8 bins: 8 pairs; from 128^3 on mostly
 // one).  64^3, 8 bins, l <= 4, all forms: 4236 us pair by pair,
-// 3864 / 3146 / 2596 / 2423 with a limit of 16 / 32 / 64 / 128 MB.
+// 3864 / 3146 / 2596 / 2423 with a limit of 16 / 32 / 64 / 128 MB.  A smaller workspace takes fewer.
 int lm_batch(const zeta_ctx* c) {
   const size_t per = sizeof(float) * static_cast<size_t>(c->ng) * (c->p.nbins + 4 * ((c->p.nbins + 3) / 4));
   const size_t fit = (static_cast<size_t>(128) << 20) / per;
@@ -36,15 +37,15 @@ int lm_batch(const zeta_ctx* c) {
   return b < pairs ? b : pairs;
 }
 // ... and of those, the pairs whose interpolated rows are held together (64 MB or one pair's rows)
-size_t rows_bytes(const zeta_ctx* c, int64_t np) {
-  const size_t one = particle_rows_bytes(c, np), all = one * lm_batch(c), cap = static_cast<size_t>(64) << 20;
+size_t rows_bytes(const zeta_ctx* c, int64_t np, int pairs) {
+  const size_t one = particle_rows_bytes(c, np), all = one * pairs, cap = static_cast<size_t>(64) << 20;
   const size_t some = all < cap ? all : cap;
   return some > one ? some : one;  // grows with np, so a workspace for more particles serves fewer
 }
 
-// Workspace regions of the full measurement for np particles (np may be 0); with backward,
-// also the regions of the gradient calls (placed after the forward ones).
-Layout layout(const zeta_ctx* c, int64_t np, bool backward = false, bool ss = false) {
+// Workspace regions of the full measurement for np particles (np may be 0), taking `pairs` (l, m) pairs
+// together; with backward, also the regions of the gradient calls (placed after the forward ones).
+Layout layout(const zeta_ctx* c, int64_t np, int pairs, bool backward = false, bool ss = false) {
   Layout L;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -55,7 +56,8 @@ Layout layout(const zeta_ctx* c, int64_t np, bool backward = false, bool ss = fa
   const size_t g = static_cast<size_t>(c->ng) * sizeof(float);
   L.delta = take(g);
   L.dhat = take(g);
-  const size_t lmb = static_cast<size_t>(lm_batch(c));
+  const size_t lmb = static_cast<size_t>(pairs);
+  L.pairs = pairs;
   L.spectra = take(g * c->p.nbins * lmb);              // plain half spectra of the C2R passes
   L.fields = take(g * 4 * ((c->p.nbins + 3) / 4) * lmb);  // bin-interleaved fields; also the assign accumulator
   L.partials = take(sizeof(double) * kMaxCtas * c->p.nbins * c->p.nbins);
@@ -67,7 +69,7 @@ Layout layout(const zeta_ctx* c, int64_t np, bool backward = false, bool ss = fa
   L.tstart = take(sizeof(int64_t) * static_cast<size_t>(c->ntiles + 1));
   L.counts = take(sizeof(int) * static_cast<size_t>(c->ntiles));
   L.orig = take(sizeof(int) * static_cast<size_t>(np));
-  L.pvals = take(rows_bytes(c, np));  // interpolated particle rows of one (l, m), or of a few
+  L.pvals = take(rows_bytes(c, np, pairs));  // interpolated particle rows of one (l, m), or of a few
   // prepared particle data (cell, offsets, weight): original order (scratch) and sorted order
   L.o_tile = take(sizeof(int) * static_cast<size_t>(np));
   L.o_cell = take(sizeof(int) * static_cast<size_t>(np));
@@ -94,10 +96,15 @@ bool tc_gram(const zeta_ctx* c) { return c->p.gram >= ZETA_GRAM_TF32 && c->p.gra
 
 int check_ctx(const zeta_ctx* c) { return c ? ZETA_OK : ZETA_EINVAL; }
 
-int need_ws(const zeta_ctx* c, int64_t np, bool backward = false, bool ss = false) {
+// The layout of a call in the caller's workspace, with as many pairs as it has room for, up to `most`.  One
+// pair is all that a call needs; zeta_workspace_bytes is the size for lm_batch pairs.
+int fit_ws(const zeta_ctx* c, int64_t np, Layout* L, int most = 1, bool backward = false, bool ss = false) {
   if (!c->ws) return ZETA_EWORKSPACE;
-  if (layout(c, np, backward, ss).total > c->ws_bytes) return ZETA_EWORKSPACE;
-  return ZETA_OK;
+  for (int pairs = most; pairs >= 1; --pairs) {
+    *L = layout(c, np, pairs, backward, ss);
+    if (L->total <= c->ws_bytes) return ZETA_OK;
+  }
+  return ZETA_EWORKSPACE;
 }
 
 template <typename T>
@@ -301,7 +308,7 @@ int zeta_destroy(zeta_ctx* c) {
 
 size_t zeta_workspace_bytes(const zeta_ctx* c, int64_t np_max, int forms) {
   if (!c || np_max < 0 || np_max > 0x7fffffffLL || forms < 0 || forms > 31) return 0;
-  return layout(c, np_max, (forms & ZETA_WS_BACKWARD) != 0, (forms & ZETA_WS_SS) != 0).total;
+  return layout(c, np_max, lm_batch(c), (forms & ZETA_WS_BACKWARD) != 0, (forms & ZETA_WS_SS) != 0).total;
 }
 
 int zeta_set_workspace(zeta_ctx* c, void* dptr, size_t bytes) {
@@ -326,8 +333,8 @@ int zeta_set_gram(zeta_ctx* c, int gram) {
 int zeta_assign(zeta_ctx* c, const float* particles, int64_t np, float* delta, double* wsum, zeta_stream stream) {
   ZK_TRY(check_ctx(c));
   if (!particles || np < 1 || np > 0x7fffffffLL || !delta) return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, 0));
-  const Layout L = layout(c, 0);
+  Layout L;
+  ZK_TRY(fit_ws(c, 0, &L));
   double* w = wsum ? wsum : at<double>(c, L.small) + kAssignScratchDoubles + 4;
   return launch_assign(c, reinterpret_cast<const float4*>(particles), np, delta, w, assign_scratch(c, L), stream);
 }
@@ -344,8 +351,8 @@ int zeta_reconstruct_alm(zeta_ctx* c, const float* delta_hat, int l, int m, int 
   if (!delta_hat || !alm || l < 0 || l > c->p.lmax || m < -l || m > l || b0 < 0 || (b0 & 3) || b1 <= b0 ||
       b1 > c->p.nbins)
     return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, 0));
-  const Layout L = layout(c, 0);
+  Layout L;
+  ZK_TRY(fit_ws(c, 0, &L));
   return launch_alm(c, reinterpret_cast<const float2*>(delta_hat), l, m, b0, b1 - b0, at<float2>(c, L.spectra), alm,
                     stream);
 }
@@ -353,8 +360,8 @@ int zeta_reconstruct_alm(zeta_ctx* c, const float* delta_hat, int l, int m, int 
 int zeta_sum_grid(zeta_ctx* c, const float* delta, const float* alm, int form, double* gram, zeta_stream stream) {
   ZK_TRY(check_ctx(c));
   if (!delta || !alm || !gram || (form != ZETA_SUM_NODE && form != ZETA_SUM_GAMMA)) return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, 0));
-  const Layout L = layout(c, 0);
+  Layout L;
+  ZK_TRY(fit_ws(c, 0, &L));
   double* part = at<double>(c, L.partials);
   if (form == ZETA_SUM_NODE)
     ZK_TRY(!tc_gram(c) ? launch_gram_node(c, delta, alm, part, stream)
@@ -369,8 +376,8 @@ int zeta_sort_particles(zeta_ctx* c, const float* particles, int64_t np, float* 
                         zeta_stream stream) {
   ZK_TRY(check_ctx(c));
   if (!particles || np < 1 || np > 0x7fffffffLL || !sorted || !tile_start) return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, np));
-  const Layout L = layout(c, np);
+  Layout L;
+  ZK_TRY(fit_ws(c, np, &L));
   return launch_sort(c, reinterpret_cast<const float4*>(particles), np, reinterpret_cast<float4*>(sorted),
                      tile_start, at<int>(c, L.counts), at<int>(c, L.orig), stream);
 }
@@ -379,8 +386,8 @@ int zeta_sum_particles(zeta_ctx* c, const float* sorted, const int64_t* tile_sta
                        const float* alm, double* gram, zeta_stream stream) {
   ZK_TRY(check_ctx(c));
   if (!sorted || !tile_start || np < 1 || !wsum || !alm || !gram) return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, np));
-  const Layout L = layout(c, np);
+  Layout L;
+  ZK_TRY(fit_ws(c, np, &L));
   double* part = at<double>(c, L.partials);
   const PartPrep q = prep_of(c, L);
   ZK_TRY(launch_prep_sorted(c, reinterpret_cast<const float4*>(sorted), np, q.s_cell, q.s_tq, stream));
@@ -391,8 +398,8 @@ int zeta_sum_particles(zeta_ctx* c, const float* sorted, const int64_t* tile_sta
 int zeta_mass_term(zeta_ctx* c, const float* delta_hat, int l, double sign, double* gram, zeta_stream stream) {
   ZK_TRY(check_ctx(c));
   if (!delta_hat || !gram || l < 0 || l > c->p.lmax || !(sign == 1.0 || sign == -1.0)) return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, 0));
-  const Layout L = layout(c, 0);
+  Layout L;
+  ZK_TRY(fit_ws(c, 0, &L));
   double* part = at<double>(c, L.partials);
   unsigned long long* hist = at<unsigned long long>(c, L.mhist);
   ZK_TRY(launch_mass_hist(c, reinterpret_cast<const float2*>(delta_hat), hist, stream));
@@ -410,9 +417,9 @@ namespace {
 // of (l, -l).  slots == false: zeta is [form][l][nb][nb], accumulated in the order 0, uniform
 // term, m = -l .. l.  slots == true: every contribution is stored in its own slot
 // [form][(lmax+1)^2 + lmax+1][nb][nb] ((l, m) at l^2 + l + m, the uniform term of l at
-// (lmax+1)^2 + l), the slots this call does not own set to zero.
+// (lmax+1)^2 + l), the slots this call does not own set to zero.  At most `most` pairs at a time.
 int measure(zeta_ctx* c, const float* particles, int64_t np, const float* delta, int forms, int lm_rank, int lm_size,
-            bool slots, double* zeta, cudaStream_t stream) {
+            bool slots, double* zeta, cudaStream_t stream, int most = kMaxLm) {
   ZK_TRY(check_ctx(c));
   if (!zeta || forms < 1 || forms > 7 || lm_size < 1 || lm_rank < 0 || lm_rank >= lm_size) return ZETA_EINVAL;
   // bfloat16 fields serve the node form alone (the other forms interpolate or integrate them)
@@ -421,8 +428,9 @@ int measure(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
   const bool want_p = forms & ZETA_SUM_PARTICLE;
   if ((want_p || !delta) && (!particles || np < 1 || np > 0x7fffffffLL)) return ZETA_EINVAL;
   const int64_t npl = want_p ? np : 0;
-  ZK_TRY(need_ws(c, npl));
-  const Layout L = layout(c, npl);
+  Layout L;
+  const int lmb = lm_batch(c);
+  ZK_TRY(fit_ws(c, npl, &L, lmb < most ? lmb : most));
   const int nb = c->p.nbins, lmax = c->p.lmax;
   const float4* parts = reinterpret_cast<const float4*>(particles);
   double* small = at<double>(c, L.small);
@@ -494,7 +502,6 @@ int measure(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
   for (int l = 0; l <= lmax; ++l)
     for (int m = -l; m <= l; ++m)
       if ((l * l + l + m) % lm_size == lm_rank) pairs.emplace_back(l, m);
-  const int lmb = lm_batch(c);
   const size_t field_floats = static_cast<size_t>(c->ng) * 4 * ((nb + 3) / 4) / (bf16f ? 2 : 1);
   const size_t one_row = want_p ? particle_rows_bytes(c, np) : 1;
   // runs a form's Gram over the pairs i0 .. i0 + k of the batch and adds the results, k as large as the
@@ -513,9 +520,9 @@ int measure(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
     }
     return ZETA_OK;
   };
-  for (size_t p0 = 0; p0 < pairs.size(); p0 += lmb) {
+  for (size_t p0 = 0; p0 < pairs.size(); p0 += L.pairs) {
     LmList lms;
-    for (size_t i = p0; i < pairs.size() && i < p0 + lmb; ++i) lms.add(pairs[i].first, pairs[i].second);
+    for (size_t i = p0; i < pairs.size() && i < p0 + L.pairs; ++i) lms.add(pairs[i].first, pairs[i].second);
     ZK_TRY(launch_alm_list(c, dhat, lms, 0, nb, at<float2>(c, L.spectra), fields, stream, bf16f));
     if (idx_node >= 0) {
       if (tc_gram(c))  // the tensor-core Grams take one pair at a time
@@ -529,7 +536,7 @@ int measure(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
       ZK_TRY(form_sums(lms, gamma_ctas(c), kMaxLm, idx_gamma, inv_ng, nullptr,
                        [&](const float* f, int k) { return launch_gram_gamma(c, prim, f, part, stream, k); }));
     if (idx_part >= 0)
-      ZK_TRY(form_sums(lms, gram_particle_parts(c), static_cast<int>(rows_bytes(c, np) / one_row), idx_part, 1.0, wsum,
+      ZK_TRY(form_sums(lms, gram_particle_parts(c), static_cast<int>(rows_bytes(c, np, L.pairs) / one_row), idx_part, 1.0, wsum,
                        [&](const float* f, int k) {
                          return launch_gram_particles(c, q.s_cell, q.s_tq, tstart, np, f, at<float>(c, L.pvals), part,
                                                       stream, k);
@@ -556,8 +563,8 @@ int zeta_xi(zeta_ctx* c, const float* particles, int64_t np, const float* delta,
   const bool want_p = forms & ZETA_SUM_PARTICLE;
   if ((want_p || !delta) && (!particles || np < 1 || np > 0x7fffffffLL)) return ZETA_EINVAL;
   const int64_t npl = want_p ? np : 0;
-  ZK_TRY(need_ws(c, npl));
-  const Layout L = layout(c, npl);
+  Layout L;
+  ZK_TRY(fit_ws(c, npl, &L));
   const int nb = c->p.nbins;
   const float4* parts = reinterpret_cast<const float4*>(particles);
   double* small = at<double>(c, L.small);
@@ -601,8 +608,8 @@ int zeta_zeta_ell_ss(zeta_ctx* c, const float* data, int64_t nd, const float* ra
   if (!data || !randoms || nd < 1 || nr < 1 || nd > 0x7fffffffLL || nr > 0x7fffffffLL || !num || !den ||
       forms < 1 || (forms & ~(ZETA_SUM_NODE | ZETA_SUM_GAMMA)))
     return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, 0, false, true));
-  const Layout L = layout(c, 0, false, true);
+  Layout L;
+  ZK_TRY(fit_ws(c, 0, &L, lm_batch(c), false, true));
   double* small = at<double>(c, L.small);
   float* dd = at<float>(c, L.delta);
   float* dr = at<float>(c, L.dss);
@@ -611,8 +618,9 @@ int zeta_zeta_ell_ss(zeta_ctx* c, const float* data, int64_t nd, const float* ra
   ZK_TRY(launch_assign(c, reinterpret_cast<const float4*>(data), nd, dd, w, sc, stream));
   ZK_TRY(launch_assign(c, reinterpret_cast<const float4*>(randoms), nr, dr, w, sc, stream));
   ZK_TRY(launch_ss_fields(c, dd, dr, stream));
-  ZK_TRY(measure(c, nullptr, 0, dd, forms, 0, 1, false, num, stream));
-  return measure(c, nullptr, 0, dr, forms, 0, 1, false, den, stream);
+  // with the pairs of this layout, so that the random grid behind its regions stays untouched
+  ZK_TRY(measure(c, nullptr, 0, dd, forms, 0, 1, false, num, stream, L.pairs));
+  return measure(c, nullptr, 0, dr, forms, 0, 1, false, den, stream, L.pairs);
 }
 
 int zeta_xi_radii(zeta_ctx* c, const float* delta_hat, int nr, const double* radii, double* xi, zeta_stream stream) {
@@ -620,8 +628,8 @@ int zeta_xi_radii(zeta_ctx* c, const float* delta_hat, int nr, const double* rad
   if (!delta_hat || !radii || !xi || nr < 1 || nr > 4096) return ZETA_EINVAL;
   for (int i = 0; i < nr; ++i)
     if (!(radii[i] >= 0) || !std::isfinite(radii[i])) return ZETA_EINVAL;
-  ZK_TRY(need_ws(c, 0));
-  const Layout L = layout(c, 0);
+  Layout L;
+  ZK_TRY(fit_ws(c, 0, &L));
   // the radii go to the device through the workspace's small scratch (after the weight sums)
   double* dr = at<double>(c, L.xi_radii);
   if (cudaMemcpyAsync(dr, radii, sizeof(double) * nr, cudaMemcpyHostToDevice, stream) != cudaSuccess)
@@ -662,13 +670,15 @@ int zeta_batch(zeta_ctx* c, const float* particles, const int64_t* offsets, int 
     if (np > np_max) np_max = np;
   }
   const int64_t npl = (forms & ZETA_SUM_PARTICLE) ? np_max : 0;
-  ZK_TRY(need_ws(c, npl));
-  // catalogues in flight: as many whole per-catalogue workspaces as the caller's holds (<= 4)
-  const size_t per_ws = layout(c, npl).total;
-  int k = static_cast<int>(c->ws_bytes / per_ws);
-  if (k > zeta_ctx::kMaxBatchStreams) k = zeta_ctx::kMaxBatchStreams;
+  Layout L1;
+  ZK_TRY(fit_ws(c, npl, &L1));
+  // catalogues in flight (<= 4): as many whole per-catalogue workspaces as the caller's holds; in a smaller one
+  // (which holds fewer pairs than zeta_workspace_bytes is for), as many as fit with a pair at a time
+  size_t per_ws = layout(c, npl, lm_batch(c)).total;
+  const size_t fit = c->ws_bytes / (c->ws_bytes >= per_ws ? per_ws : L1.total);
+  int k = fit < zeta_ctx::kMaxBatchStreams ? static_cast<int>(fit) : zeta_ctx::kMaxBatchStreams;
   if (k > ncat) k = ncat;
-  if (k < 1) k = 1;
+  if (c->ws_bytes < per_ws) per_ws = c->ws_bytes / k / kAlign * kAlign;
   std::vector<int64_t> key = {static_cast<int64_t>(reinterpret_cast<uintptr_t>(particles)),
                               static_cast<int64_t>(reinterpret_cast<uintptr_t>(zeta)), forms, ncat, k};
   key.insert(key.end(), offsets, offsets + ncat + 1);
@@ -738,8 +748,8 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
   ZK_TRY(check_ctx(c));
   if (!particles || np < 1 || np > 0x7fffffffLL || forms < 1 || forms > 7) return ZETA_EINVAL;
   const bool want_p = forms & ZETA_SUM_PARTICLE;
-  ZK_TRY(need_ws(c, want_p ? np : 0));
-  const Layout L = layout(c, want_p ? np : 0);
+  Layout L;
+  ZK_TRY(fit_ws(c, want_p ? np : 0, &L));
   const float4* parts = reinterpret_cast<const float4*>(particles);
   double* small = at<double>(c, L.small);
   double* wsum = small + kAssignScratchDoubles + 4;
@@ -940,8 +950,8 @@ int zeta_backward_node(zeta_ctx* c, const float* delta, const double* weights, f
   ZK_TRY(check_ctx(c));
   if (!delta || !weights || !grad) return ZETA_EINVAL;
   if (c->p.tophat_primary > 0) return ZETA_ENOTSUP;
-  ZK_TRY(need_ws(c, 0, true));
-  const Layout L = layout(c, 0, true);
+  Layout L;
+  ZK_TRY(fit_ws(c, 0, &L, 1, true));
   const int nb = c->p.nbins;
   float* S = at<float>(c, L.wts);
   ZK_TRY(upload_weights(c, weights, S, stream));
@@ -972,8 +982,8 @@ int zeta_backward_particles(zeta_ctx* c, const float* particles, int64_t np, con
   if (!particles || np < 1 || np > 0x7fffffffLL || !weights || !grad) return ZETA_EINVAL;
   if (c->p.tophat_primary > 0) return ZETA_ENOTSUP;
   if (c->p.dsup == 3) return ZETA_ENOTSUP;  // the Daubechies function has no derivative to move points with
-  ZK_TRY(need_ws(c, np, true));
-  const Layout L = layout(c, np, true);
+  Layout L;
+  ZK_TRY(fit_ws(c, np, &L, 1, true));
   const int nb = c->p.nbins;
   float* S = at<float>(c, L.wts);
   ZK_TRY(upload_weights(c, weights, S, stream));
