@@ -567,7 +567,8 @@ __global__ void __launch_bounds__(kThreads)
   cta_store<NBP>(g, red, nb, partials + static_cast<long long>(blockIdx.x) * nb * nb);
 }
 
-// Gamma form of the cubic B-spline and Daubechies bases for up to 20 bins: the batches, their order and all
+// Gamma form of the cubic B-spline and Daubechies bases for up to 20 bins (Daubechies with 17 to 20 only in
+// launches of a CTA per SM or fewer: gamma_impl): the batches, their order and all
 // arithmetic of k_gram_gamma, with the x pass taken out of the batch.  A tile is walked layer by layer and
 // row by row; the x-filtered values of the D stencil rows of the current row of cells (8 K points each, D
 // planes) are kept in a ring, and going to the next row filters one new stencil row per plane instead of
@@ -1155,11 +1156,21 @@ int gamma_impl(const zeta_ctx* c, const float* delta, const float* alm, double* 
     const size_t main = GammaLin<NBP>::BYTES, sm = main > red_bytes<NBP>() ? main : red_bytes<NBP>();
     if (prep(k_gram_gamma_lin<NBP>, sm)) return ZETA_ECUDA;
     k_gram_gamma_lin<NBP><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
-  } else if constexpr (D > 2 && NBP <= 20) {
+    return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
+  }
+  if constexpr (D > 2 && NBP <= 20) {
+    // The row ring pays as long as it costs no CTA of an SM: where two fit (every case but the Daubechies basis
+    // with 17 to 20 bins, whose ring takes 131 KB), or where there is one CTA per SM or fewer anyway.
+    // Daubechies, 20 bins, us, k_gram_gamma / rows: 32^3 648 / 473, 64^3 1843 / 1856, 128^3 12334 / 13321.
+    // More bins would leave one CTA per SM for D = 4 as well.
     const size_t main = GammaRows<NBP, D>::BYTES, sm = main > red_bytes<NBP>() ? main : red_bytes<NBP>();
-    if (prep(k_gram_gamma_rows<NBP, D>, sm)) return ZETA_ECUDA;
-    k_gram_gamma_rows<NBP, D><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
-  } else {  // more bins; with D > 2 their row ring would leave one CTA per SM
+    if (2 * (sm + 1024) <= 228 * 1024 || static_cast<long long>(grid.x) * nlm <= c->num_sms) {
+      if (prep(k_gram_gamma_rows<NBP, D>, sm)) return ZETA_ECUDA;
+      k_gram_gamma_rows<NBP, D><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
+      return cudaGetLastError() == cudaSuccess ? ZETA_OK : ZETA_ECUDA;
+    }
+  }
+  if constexpr (D > 2 || NBP > 12) {
     const size_t sm = smem_gamma<NBP, D>();
     if (prep(k_gram_gamma<NBP, D>, sm)) return ZETA_ECUDA;
     k_gram_gamma<NBP, D><<<grid, kThreads, sm, s>>>(delta, f4, c->ng, c->n, c->p.nbins, c->d_gq, partials);
