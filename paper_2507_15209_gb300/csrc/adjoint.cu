@@ -54,8 +54,10 @@ __device__ __forceinline__ int cell_t(float x, const CellScale& cs, int n, float
 }
 
 // q += sum S a a and the fields replaced by h = 2 delta S a, two points per thread so that each float4 of S
-// read from shared memory serves eight multiply-adds.  Bound: HBM (fields read and
-// written) and shared-memory reads.  256^3, 10 bins: 550 us, 3.3 TB/s.
+// read from shared memory serves eight multiply-adds.  The loop over the groups of h is rolled (unrolled, S
+// fills the registers and spills).  Bound: HBM, the fields read once and written once.  256^3, us, with 8, 10,
+// 16, 20, 28 and 32 bins: 203, 278, 418, 470, 772, 914 (one point per thread, both loops unrolled: 330, 703,
+// 745, 934, 1348, 1374; each group's values read a second time, which missed L1: 306, 546, 745, 978, 1408, 902).
 template <int NBP>
 __global__ void __launch_bounds__(kAT) k_adj_node(const float* __restrict__ delta, float4* __restrict__ f4, long long ng,
                                                   int nb, const float* __restrict__ S, float* __restrict__ q) {
@@ -86,9 +88,14 @@ __global__ void __launch_bounds__(kAT) k_adj_node(const float* __restrict__ delt
 #pragma unroll 1
     for (int g = 0; g < G; ++g) {
       float h[P][4];
-      float4 own[P];  // this group's values once more (a itself is indexed by constants only)
+      float4 own[P];  // this group's values, by selects (a is indexed by constants only)
 #pragma unroll
-      for (int u = 0; u < P; ++u) own[u] = f4[g * ng + i0 + u * kAT];
+      for (int u = 0; u < P; ++u) {
+        own[u] = make_float4(a[u][0], a[u][1], a[u][2], a[u][3]);
+#pragma unroll
+        for (int g2 = 1; g2 < G; ++g2)
+          if (g == g2) own[u] = make_float4(a[u][4 * g2], a[u][4 * g2 + 1], a[u][4 * g2 + 2], a[u][4 * g2 + 3]);
+      }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int b = 4 * g + j;
