@@ -749,7 +749,7 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
   if (!particles || np < 1 || np > 0x7fffffffLL || forms < 1 || forms > 7) return ZETA_EINVAL;
   const bool want_p = forms & ZETA_SUM_PARTICLE;
   Layout L;
-  ZK_TRY(fit_ws(c, want_p ? np : 0, &L));
+  ZK_TRY(fit_ws(c, want_p ? np : 0, &L, lm_batch(c)));
   const float4* parts = reinterpret_cast<const float4*>(particles);
   double* small = at<double>(c, L.small);
   double* wsum = small + kAssignScratchDoubles + 4;
@@ -759,7 +759,7 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
   double* part = at<double>(c, L.partials);
   float4* sorted = at<float4>(c, L.sorted);
   int64_t* tstart = at<int64_t>(c, L.tstart);
-  // representative data: this catalogue's fields for one (l, m)
+  // representative data: this catalogue's fields for one (l, m), as many times as a launch takes pairs
   const PartPrep q = prep_of(c, L);
   ZK_TRY(launch_assign(c, parts, np, dl, wsum, assign_scratch(c, L), stream));
   ZK_TRY(launch_r2c(c, dl, dhat, stream));
@@ -769,17 +769,33 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
     ZK_TRY(launch_mass_hist(c, dhat, hist, stream));
   }
   const int l = c->p.lmax < 2 ? c->p.lmax : 2;
-  ZK_TRY(launch_alm(c, dhat, l, 0, 0, c->p.nbins, at<float2>(c, L.spectra), fields, stream));
+  LmList lms;
+  for (int i = 0; i < L.pairs; ++i) lms.add(l, 0);
+  ZK_TRY(launch_alm_list(c, dhat, lms, 0, c->p.nbins, at<float2>(c, L.spectra), fields, stream));
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return ZETA_ECUDA;
+  // pairs (multipoles of the uniform term) that a launch of the measurement takes at the present grid sizes
+  auto taken = [&](int kind) -> int {
+    const int parts = kind == GK_GAMMA  ? gamma_ctas(c)
+                      : kind == GK_PART ? gram_particle_parts(c)
+                      : kind == GK_MASS ? mass_ctas(c)
+                                        : gram_ctas(c, kind);
+    int most = kind == GK_TC ? 1 : kind == GK_MASS ? c->p.lmax + 1 : L.pairs;
+    if (kind == GK_PART) {
+      const int rows = static_cast<int>(rows_bytes(c, np, L.pairs) / particle_rows_bytes(c, np));
+      most = most < rows ? most : rows;
+    }
+    return most < kMaxCtas / parts ? most : kMaxCtas / parts;
+  };
   auto run = [&](int kind) -> int {
+    const int k = taken(kind);
     switch (kind) {
-      case GK_NODE: return launch_gram_node(c, dl, fields, part, stream);
+      case GK_NODE: return launch_gram_node(c, dl, fields, part, stream, false, k);
       case GK_TC: return launch_gram_node_tc(c, dl, fields, part, stream);
-      case GK_GAMMA: return launch_gram_gamma(c, dl, fields, part, stream);
+      case GK_GAMMA: return launch_gram_gamma(c, dl, fields, part, stream, k);
       case GK_PART:
-        return launch_gram_particles(c, q.s_cell, q.s_tq, tstart, np, fields, at<float>(c, L.pvals), part, stream);
-      default: return launch_mass(c, hist, l, part, stream);
+        return launch_gram_particles(c, q.s_cell, q.s_tq, tstart, np, fields, at<float>(c, L.pvals), part, stream, k);
+      default: return launch_mass(c, hist, 0, part, stream, k);
     }
   };
   std::vector<int> kinds;
@@ -790,7 +806,7 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
     kinds.push_back(GK_MASS);
   }
   int rc = ZETA_OK;
-  // one warm-up call, then the faster of two timed blocks of three calls (-1 on error)
+  // one warm-up call, then the faster of two timed blocks of three calls, per pair (-1 on error)
   auto time_ms = [&](int kind) -> float {
     if ((rc = run(kind)) != ZETA_OK) return -1.f;
     float best_ms = 1e30f;
@@ -806,7 +822,7 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
       cudaEventElapsedTime(&ms, e0, e1);
       if (ms < best_ms) best_ms = ms;
     }
-    return best_ms;
+    return best_ms / taken(kind);
   };
   const int cand[] = {1, 2, 3, 4, 6, 8};
   for (int kind : kinds) {
@@ -844,11 +860,11 @@ int zeta_autotune(zeta_ctx* c, const float* particles, int64_t np, int forms, ze
   // passes cost the same under either shape of the pass being chosen)
   float2* spec = at<float2>(c, L.spectra);
   auto time_alm = [&]() -> float {
-    if ((rc = launch_alm(c, dhat, l, 0, 0, c->p.nbins, spec, fields, stream)) != ZETA_OK) return -1.f;
+    if ((rc = launch_alm_list(c, dhat, lms, 0, c->p.nbins, spec, fields, stream)) != ZETA_OK) return -1.f;
     float best_ms = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
       cudaEventRecord(e0, stream);
-      for (int r = 0; r < 2 && rc == ZETA_OK; ++r) rc = launch_alm(c, dhat, l, 0, 0, c->p.nbins, spec, fields, stream);
+      for (int r = 0; r < 2 && rc == ZETA_OK; ++r) rc = launch_alm_list(c, dhat, lms, 0, c->p.nbins, spec, fields, stream);
       cudaEventRecord(e1, stream);
       if (rc != ZETA_OK || cudaEventSynchronize(e1) != cudaSuccess) {
         rc = rc ? rc : ZETA_ECUDA;
