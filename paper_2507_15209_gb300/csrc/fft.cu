@@ -829,13 +829,10 @@ int alm_z_pass(const zeta_ctx* c, const float2* dhat, const LmList& lms, int b0,
       return check_launch();
     }
   }
+  if (lms.n != 1) return ZETA_EINVAL;  // grids above 128^3 take one pair (lm_batch)
   if (set_smem(k_alm_z<N, T, false>, smz)) return ZETA_ECUDA;
-  for (int i = 0; i < lms.n; ++i) {
-    LmList one;
-    one.add(lms.l[i], lms.m[i]);
-    k_alm_z<N, T, false><<<dim3(NC / T, N / 2 + 1), AlmZ<N, T>::NT, smz, s>>>(
-        dhat, spec + i * nf * fstride, fstride, nf, jt4 + lms.l[i] * jstride, nbp4, one, jstride, nf, c->d_tw, c->d_phi);
-  }
+  k_alm_z<N, T, false><<<dim3(NC / T, N / 2 + 1), AlmZ<N, T>::NT, smz, s>>>(
+      dhat, spec, fstride, nf, jt4 + lms.l[0] * jstride, nbp4, lms, jstride, nf, c->d_tw, c->d_phi);
   return check_launch();
 }
 
@@ -863,11 +860,9 @@ int alm_x_pass(const zeta_ctx* c, int nlm, int nf, const float2* spec, float* ou
       constexpr int XT = kX4Threads;
       using Y = X4v<N, XT>;
       const dim3 grid(N * N / Y::RB, ng4);
-      const size_t per = static_cast<size_t>(ng4) * N * N * N * (bf16 ? 2 : 4);  // floats of one pair's fields
+      if (nlm != 1) return ZETA_EINVAL;  // one pair at a time on these grids (lm_batch)
       if (set_smem(bf16 ? k_c2r_x4v<N, XT, true> : k_c2r_x4v<N, XT, false>, Y::SMEM)) return ZETA_ECUDA;
-      for (int i = 0; i < nlm; ++i)
-        (bf16 ? k_c2r_x4v<N, XT, true> : k_c2r_x4v<N, XT, false>)<<<grid, XT, Y::SMEM, s>>>(
-            spec + i * nf * fstride, fstride, nf, out + i * per, c->d_tw);
+      (bf16 ? k_c2r_x4v<N, XT, true> : k_c2r_x4v<N, XT, false>)<<<grid, XT, Y::SMEM, s>>>(spec, fstride, nf, out, c->d_tw);
       return check_launch();
     }
   }
