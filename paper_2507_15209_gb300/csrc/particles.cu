@@ -629,7 +629,7 @@ bool halo_map(const zeta_ctx* c, const float* fields, int ngroups, CUtensorMap* 
   static const Encode encode = [] {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess ||
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
         q != cudaDriverEntryPointSuccess)
       fn = nullptr;
     return reinterpret_cast<Encode>(fn);
