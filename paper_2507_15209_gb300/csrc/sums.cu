@@ -1149,7 +1149,7 @@ int node_impl(const zeta_ctx* c, const float* delta, const float* alm, double* p
 template <int NBP, int D>
 int gamma_impl(const zeta_ctx* c, const float* delta, const float* alm, double* partials, cudaStream_t s, int nlm) {
   StageScope prof(c, ST_GRAM_GAMMA, 1, s);
-  if (c->gamma_q != GammaShape<NBP, D>::K) return ZETA_EINVAL;
+  if (c->gamma_q != (D == 2 ? 2 : 5)) return ZETA_EINVAL;  // GammaShape::K
   const float4* f4 = reinterpret_cast<const float4*>(alm);
   const dim3 grid(gamma_ctas(c), nlm);
   if constexpr (D == 2 && NBP <= 12) {  // 128^3, 12 bins: 634 us with k_gram_gamma, 554; more bins: see GammaLin
