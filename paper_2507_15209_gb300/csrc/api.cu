@@ -368,8 +368,8 @@ int zeta_sum_grid(zeta_ctx* c, const float* delta, const float* alm, int form, d
                        : launch_gram_node_tc(c, delta, alm, part, stream));
   else
     ZK_TRY(launch_gram_gamma(c, delta, alm, part, stream));
-  return launch_reduce(c, part,
-                       form == ZETA_SUM_NODE ? gram_ctas(c, tc_gram(c) ? GK_TC : GK_NODE) : gamma_ctas(c), 1.0 / static_cast<double>(c->ng), nullptr, gram, stream);
+  const int parts = form == ZETA_SUM_NODE ? gram_ctas(c, tc_gram(c) ? GK_TC : GK_NODE) : gamma_ctas(c);
+  return launch_reduce(c, part, parts, 1.0 / static_cast<double>(c->ng), nullptr, gram, stream);
 }
 
 int zeta_sort_particles(zeta_ctx* c, const float* particles, int64_t np, float* sorted, int64_t* tile_start,

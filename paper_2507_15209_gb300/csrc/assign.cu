@@ -6,8 +6,8 @@
 //   eps_bar = W / N_g.
 // Contributions are scattered as 64-bit fixed point (scale 2^k with k chosen from sum |w|
 // so no cell can overflow), so the result does not depend on the order of the atomics.
-// The cell and in-cell offset of each particle are computed in float64 so that a float32
-// position of a 512^3 grid keeps its full in-cell resolution.
+// The cell and in-cell offset of each particle are those of the float64 formula, bit for bit (formed with
+// integers, cell.cuh), so that a float32 position of a 512^3 grid keeps its full in-cell resolution.
 //
 // Tiling: particles are counted into 8x8x8-cell tiles, prefix-summed, scattered, and each
 // tile's list is put back into original order, so particle-form sums are reproducible.
@@ -135,8 +135,9 @@ __global__ void __launch_bounds__(256) k_weight_partials(const float4* __restric
 }
 
 // out[0] = W, out[1] = sum |w|, out[2] = fixed-point scale 2^k (sum |w| * 2^k < 2^62), out[4] = the factor
-// N_g / (W 2^k) of the contrast and out[3] the same as a pair of float32 (NaN when the pair cannot hold it).  One CTA: thread t adds the partials t, t + 256, ..., then the CTA adds its threads in a fixed
-// order (one thread adding the 1024 partials in turn took 107 us, this 5 us).
+// N_g / (W 2^k) of the contrast and out[3] the same as a pair of float32 (NaN when the pair cannot hold it).
+// One CTA: thread t adds the partials t, t + 256, ..., then the CTA adds its threads in a fixed order (one
+// thread adding the 1024 partials in turn took 107 us, this 5 us).
 __global__ void __launch_bounds__(256) k_weight_final(const double* __restrict__ part, int nparts, double ng,
                                                       double* __restrict__ out, double* __restrict__ wsum) {
   double a = 0.0, b = 0.0;
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(256) k_weight_final(const double* __restrict__
   if (wsum) *wsum = a;
 }
 
-// The float64 cell arithmetic of a particle, done once per catalogue: cell (linear index
+// The cell arithmetic of a particle (cell_of), done once per catalogue: cell (linear index
 // z n^2 + y n + x), in-cell offsets t in [0, 1) and the weight (0 for a non-finite particle,
 // which sits in cell 0 with t = 0 and so contributes nothing anywhere).
 __device__ __forceinline__ void prep_one(float4 q, const CellScale& cs, int n, int shift, int& cell, float4& tq,

@@ -219,7 +219,7 @@ int launch_assign(const zeta_ctx* c, const float4* parts, int64_t np, float* del
                   const AssignScratch& a, cudaStream_t s);
 int launch_wsum(const zeta_ctx* c, const float4* parts, int64_t np, double* wsum, double* scratch, cudaStream_t s);
 constexpr int kAssignScratchDoubles = 2 * 1024 + 6;
-// Per-particle data computed once per catalogue with the float64 cell arithmetic, so the kernels
+// Per-particle data computed once per catalogue (the cell arithmetic of cell.cuh), so the kernels
 // that run per (l, m) need none: the cell (linear index z n^2 + y n + x) and (t_x, t_y, t_z, w),
 // the in-cell offsets and the weight (0 for a non-finite particle).  o_*: original order
 // (scratch, with the tile of each particle), s_*: sorted order.
