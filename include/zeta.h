@@ -318,9 +318,9 @@ int zeta_backward_particles(zeta_ctx* ctx, const float* particles, int64_t np, c
 int zeta_batch(zeta_ctx* ctx, const float* particles, const int64_t* offsets, int ncat, int forms, double* zeta,
                zeta_stream stream);
 
-/* Autotuner: on this catalogue, times the Gram kernels that `forms` uses at persistent grid
- * sizes of 1, 2, 3, 4, 6 and 8 CTAs per SM and keeps the fastest for each kernel (used by all
- * later calls); with the particle form it then picks the staging threshold of
+/* Autotuner: on this catalogue, times the Gram kernels that `forms` uses, in launches of as many
+ * (l, m) pairs as a measurement in this workspace takes, at persistent grid sizes of 1, 2, 3, 4, 6
+ * and 8 CTAs per SM and keeps the fastest for each kernel (used by all later calls); with the particle form it then picks the staging threshold of
  * zeta_set_staging the same way; last it picks the tile shape of each field-reconstruction
  * pass (zeta_set_shapes).  Synchronises the stream; overwrites the workspace. */
 int zeta_autotune(zeta_ctx* ctx, const float* particles, int64_t np, int forms, zeta_stream stream);

@@ -175,10 +175,13 @@ __global__ void __launch_bounds__(kAT) k_adj_mass(const float2* __restrict__ dha
 // 64 contiguous bytes.  Per bin group the lanes sum w v and the parts of its gradient over their nodes, then
 // reduce-scatter: lane i holds f and grad f of bin 4 g + i.  c = (2 w_p / W) S f takes f from the other
 // lanes by shuffles; the direct term sum_b c_b grad f_b is added to the particle's slot; and c is
-// scattered with the assignment stencil by float4 atomics.  Bound: L2 atomics and gathers.  256^3, 1M
-// particles, 10 bins, D = 4: 2167 us with one thread per particle and bin group (values and gradients
-// through shared memory), 974 with
-// the sixteen rows unrolled (spills at two CTAs per SM), about 835 with rolled layers and three.
+// scattered with the assignment stencil by float4 atomics.  Bound: the latency of the gathers and atomics at 24
+// warps per SM (10 bins: long scoreboard 13.9 cycles an instruction, L1 74 % and L2 59 % busy).  256^3, 1M
+// particles, D = 4, us, with 10, 16, 20
+// and 32 bins: 852, 1198, 1525, 2785 (one thread per particle and bin group, values and gradients through
+// shared memory: 2179, 2846, 3403, 5638).  Three CTAs per SM cost spills of 44 to 124 bytes a thread from 13 bins
+// on and are still faster than two, but for 32 bins: 930, 1243, 1560, 2714 with two.  With the sixteen rows
+// unrolled, two CTAs and 10 bins: 974.
 template <int NBP, int D>
 __global__ void __launch_bounds__(kAT, 3)
     k_adj_points(const int* __restrict__ s_cell, const float4* __restrict__ s_tq, const int* __restrict__ sidx,

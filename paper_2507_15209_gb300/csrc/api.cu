@@ -26,9 +26,9 @@ struct Layout {
 
 // (l, m) pairs that a measurement takes together.  On small grids every kernel of one pair is a few
 // microseconds of latency on a machine that is mostly idle, so the pairs share launches as long as their
-// spectra and fields stay within 128 MB, an L2's worth (64^3 with 8 bins: 8 pairs; from 128^3 on mostly
-// one).  64^3, 8 bins, l <= 4, all forms: 4236 us pair by pair,
-// 3864 / 3146 / 2596 / 2423 with a limit of 16 / 32 / 64 / 128 MB.  A smaller workspace takes fewer.
+// spectra and fields stay within 128 MB, an L2's worth (64^3 with 8 bins: 8 pairs; 128^3: 3 with one bin, 2 with
+// up to 4; else one).  64^3, 8 bins, l <= 4, all forms: 4236 us pair by pair, 3864 / 3146 / 2596 / 2423 with a
+// limit of 16 / 32 / 64 / 128 MB.  A smaller workspace takes fewer.
 int lm_batch(const zeta_ctx* c) {
   const size_t per = sizeof(float) * static_cast<size_t>(c->ng) * (c->p.nbins + 4 * ((c->p.nbins + 3) / 4));
   const size_t fit = (static_cast<size_t>(128) << 20) / per;

@@ -721,10 +721,12 @@ __global__ void __launch_bounds__(kThreads)
 // Gamma form of the linear B-spline: the batches (32 cells, 8 points each), their order and all arithmetic of
 // k_gram_gamma, but one thread takes a cell's eight nodes of one channel through the three passes in
 // registers (lanes along x, so the loads are coalesced), and two batches share a round: two barriers per
-// two batches instead of four per batch, and no pass buffers.  us per (l, m), k_gram_gamma -> here: 3 bins at
-// 32^3 53 -> 39; 8 at 64^3 89 -> 61, at 256^3 3810 -> 1983.
+// two batches instead of four per batch, and no pass buffers.  us per (l, m), k_gram_gamma -> here: 4 bins at
+// 32^3 52 -> 30; 8 at 64^3 88 -> 59, at 256^3 3826 -> 1992.
 // Up to 12 bins the channels of a round (bins in fours, and delta) fit its threads; with more, a mostly idle
 // second pass over them makes it slower on large grids (256^3: 15 bins 5810 -> 6660, 20 bins 7210 -> 7545).
+// With 9 to 12 bins its registers leave one CTA per SM where k_gram_gamma has two, and it is still the faster
+// one: 12 bins at 64^3 111 -> 92, 128^3 636 -> 557, 256^3 4854 -> 4208.
 template <int NBP>
 struct GammaLin {
   static constexpr int BATCHES = 2;
@@ -1043,11 +1045,10 @@ __global__ void k_reduce_lm(const double* __restrict__ slots, int nforms, int pa
 // W_p(k) over the non-Nyquist modes, which depends on the mode only through |n|^2 apart from
 // Phi-hat: so the per-|n|^2 sums H of (1 or 2) |delta_hat|^2 Phi-hat (the fixed-point histogram of
 // the uniform term, with Phi-hat as its per-axis table) give every bin, and any radius, as one
-// sum over the 3 (n/2 - 1)^2 + 1 values of |n|^2.  One CTA per output value; each thread sums
-// a fixed stride of |n|^2 in float64 and the CTA reduces in a fixed order.
+// sum over the 3 (n/2 - 1)^2 + 1 values of |n|^2.  Each output is split over gridDim.y CTAs; a thread sums a
+// fixed stride of |n|^2 in float64, the CTA adds its threads in a fixed order, and k_xi_final the CTAs.
 // mode 0: out[b] for the bins, radial factor from the window table (l = 0 row);
 // mode 1: out[i] for radii[i], radial factor j_0(k r_i) W_TH(k rsec).
-// Each output is split over gridDim.y CTAs (a stride of |n|^2 each) whose partial sums k_xi_final adds.
 __global__ void __launch_bounds__(256) k_xi_hist(const unsigned long long* __restrict__ hist, long long nn2,
                                                  const float* __restrict__ jt0, int nbp, const float* __restrict__ wprim,
                                                  double ng, double kunit, const double* __restrict__ radii,
